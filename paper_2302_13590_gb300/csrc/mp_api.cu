@@ -310,6 +310,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     const size_t o_delr = off; off = align256(off + sizeof(double) * nc);
     const size_t o_delc = off; off = align256(off + sizeof(double) * nr);
     const size_t o_dz = off; off = align256(off + sizeof(double) * nl);
+    const size_t o_ax = off; off = align256(off + sizeof(AxisCell) * (nc + nr + nl));
     const size_t o_xf = off; off = align256(off + sizeof(double) * (nc + 1));
     const size_t o_yf = off; off = align256(off + sizeof(double) * (nr + 1));
     const size_t o_zf = off; off = align256(off + sizeof(double) * (nl + 1));
@@ -341,6 +342,19 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     zf[0] = d->origin[2];
     for (long long a = 0; a < nl; ++a) zf[a + 1] = zf[a] + d->dz[a];
 
+    std::vector<AxisCell> axc;
+    axc.reserve((size_t)(nc + nr + nl));
+    int no_screen = 0;
+    auto add_axis = [&](const double* D, long long m) {
+        for (long long a = 0; a < m; ++a) {
+            axc.push_back(AxisCell{D[a], host_f32_trunc(D[a]), 0.0f});
+            if (D[a] > SCREEN_MAX_D) no_screen = 1;
+        }
+    };
+    add_axis(d->delr, nc);
+    add_axis(d->delc, nr);
+    add_axis(d->dz, nl);
+
     cudaStream_t s = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaStreamCreate"));
@@ -366,6 +380,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
         (e = cudaMemcpyAsync(buf + o_delr, d->delr, sizeof(double) * nc, h2d, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(buf + o_delc, d->delc, sizeof(double) * nr, h2d, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(buf + o_dz, d->dz, sizeof(double) * nl, h2d, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(buf + o_ax, axc.data(), sizeof(AxisCell) * axc.size(), h2d, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(buf + o_xf, xf.data(), sizeof(double) * (nc + 1), h2d, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(buf + o_yf, yf.data(), sizeof(double) * (nr + 1), h2d, s)) != cudaSuccess ||
         (e = cudaMemcpyAsync(buf + o_zf, zf.data(), sizeof(double) * (nl + 1), h2d, s)) != cudaSuccess ||
@@ -392,6 +407,8 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     f->d.delr = reinterpret_cast<double*>(buf + o_delr);
     f->d.delc = reinterpret_cast<double*>(buf + o_delc);
     f->d.dz = reinterpret_cast<double*>(buf + o_dz);
+    f->d.ax = reinterpret_cast<AxisCell*>(buf + o_ax);
+    f->d.no_screen = no_screen;
     f->d.xf = reinterpret_cast<double*>(buf + o_xf);
     f->d.yf = reinterpret_cast<double*>(buf + o_yf);
     f->d.zf = reinterpret_cast<double*>(buf + o_zf);
@@ -471,10 +488,13 @@ int mp_usg_field_load(mp_ctx* ctx, const mp_usg_desc* d, mp_field** out)
         if (d->face_off[k + 1] < d->face_off[k]) return fail(MP_ERR_SHAPE, "mp_usg_field_load: face_off decreases");
     const long long ns = d->face_off[6 * nc];
     if (ns > 0x7fffffffLL) return fail(MP_ERR_SHAPE, "mp_usg_field_load: more than 2^31 sub-faces");
+    int no_screen = 0;
     for (long long c = 0; c < nc; ++c) {
         for (int a = 0; a < 6; ++a)
             if (!std::isfinite(d->box[6 * c + a]) || (a >= 3 && !(d->box[6 * c + a] > 0.0)))
                 return fail(MP_ERR_NONFINITE, "mp_usg_field_load: box must be finite with sizes > 0");
+        for (int a = 3; a < 6; ++a)
+            if (d->box[6 * c + a] > mp::SCREEN_MAX_D) no_screen = 1;
         const int8_t ib = d->ibound[c];
         if (ib < -1 || ib > 2) return fail(MP_ERR_INVALID_ARG, "mp_usg_field_load: ibound outside {-1, 0, 1, 2}");
         if ((ib == 1 || ib == 2) && !(d->porosity[c] > 0.0 && d->porosity[c] <= 1.0))
@@ -510,6 +530,7 @@ int mp_usg_field_load(mp_ctx* ctx, const mp_usg_desc* d, mp_field** out)
         for (int a = 0; a < 4; ++a) sub[e].rect[a] = d->rect[4 * e + a];
     }
     mp::DevUsg u{};
+    u.no_screen = no_screen;
     u.ncell = nc;
     u.nsub = ns;
     u.cell = reinterpret_cast<mp::UsgCell*>(buf + o_cell);

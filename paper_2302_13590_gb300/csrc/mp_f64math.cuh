@@ -55,10 +55,56 @@ __device__ __forceinline__ long long dkey(double v)
 }
 // a >= b for non-NaN a, b
 __device__ __forceinline__ bool ge_d(double a, double b) { return dkey(a) >= dkey(b); }
-// v < +inf (false for +inf and NaN)
-__device__ __forceinline__ bool lt_inf(double v)
+
+// The two 32-bit words of v, opaque to the optimiser like bits(): most tests
+// below need one of them, or one three-input operation on both.
+__device__ __forceinline__ void words(double v, unsigned& lo, unsigned& hi)
 {
-    return (bits(v) & 0x7fffffffffffffffLL) < 0x7ff0000000000000LL || bits(v) == (long long)0xfff0000000000000ULL;
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "d"(v));
+}
+__device__ __forceinline__ unsigned hi_abs(unsigned hi) { return hi & 0x7fffffffu; }
+// v == 0 (either sign) from its words
+__device__ __forceinline__ bool zero_w(unsigned lo, unsigned hi) { return (lo | hi_abs(hi)) == 0u; }
+
+// a key of times whose signed order is the IEEE order, -0 apart (below +0):
+// a >= b exactly when tkey(a) >= tkey(b); three integer operations
+__device__ __forceinline__ long long tkey(double v)
+{
+    unsigned lo, hi;
+    words(v, lo, hi);
+    const unsigned n = (unsigned)((int)hi >> 31);
+    return (long long)(((unsigned long long)(hi ^ (n >> 1)) << 32) | (lo ^ n));
+}
+// the key of a bound that may be -0, to compare sums of times with (those
+// are not -0)
+__device__ __forceinline__ long long bound_key(double v) { return tkey(eq0(v) ? 0.0 : v); }
+
+// f32_trunc from the words where 2^-126 <= |x| < 2^128 (elsewhere: some
+// value): the exponent's low nine bits and the top 23 fraction bits come out
+// of one funnel shift, the rebias is one addition
+__device__ __forceinline__ float trunc_normal(unsigned lo, unsigned hi)
+{
+    const unsigned t = __funnelshift_l(lo, hi, 3) + 0x40000000u;   // - (896 mod 512) << 23
+    return __uint_as_float(t | (hi & 0x80000000u));
+}
+// f32_trunc where |x| < 2^128 (below 2^-126: a signed zero)
+__device__ __forceinline__ float trunc_small(unsigned lo, unsigned hi)
+{
+    const unsigned t = __funnelshift_l(lo, hi, 3) + 0x40000000u;
+    return __uint_as_float((hi_abs(hi) < 0x38100000u ? 0u : t) | (hi & 0x80000000u));
+}
+// the same for x >= 0 (or -0: zero)
+__device__ __forceinline__ float trunc_pos(unsigned lo, unsigned hi)
+{
+    const unsigned t = __funnelshift_l(lo, hi, 3) + 0x40000000u;
+    return __uint_as_float((int)hi < 0x38100000 ? 0u : t);
+}
+// neither infinite nor NaN
+__device__ __forceinline__ bool is_finite(double v)
+{
+    unsigned lo, hi;
+    words(v, lo, hi);
+    return hi_abs(hi) < 0x7ff00000u;
 }
 
 // -v (the sign bit flipped, as IEEE negation)
@@ -146,8 +192,14 @@ __device__ __forceinline__ double f2d_pos(float f)
 __device__ __forceinline__ double f2d_normal(float f)
 {
     const unsigned fb = __float_as_uint(f);
-    return __longlong_as_double(((long long)(fb >> 31) << 63) | ((long long)(((fb >> 23) & 0xffu) + 896u) << 52) |
-                                ((long long)(fb & 0x7fffffu) << 29));
+    // sign | (exponent + 896) | top 20 fraction bits: an arithmetic shift by 3, the copies of the sign masked
+    return __hiloint2double((int)((((unsigned)((int)fb >> 3)) & 0x8fffffffu) + 0x38000000u), (int)(fb << 29));
+}
+// the same for f > 0
+__device__ __forceinline__ double f2d_normal_pos(float f)
+{
+    const unsigned fb = __float_as_uint(f);
+    return __hiloint2double((int)((fb >> 3) + 0x38000000u), (int)(fb << 29));
 }
 
 // d / v as d times 1 / v: the IEEE FP32 reciprocal y0 of the truncated v
@@ -161,9 +213,10 @@ static __device__ __noinline__ double div_ieee(double a, double b) { return a / 
 
 __device__ __forceinline__ double f64_div(double d, double v)
 {
-    const int e = (int)((bits(v) >> 52) & 0x7ff) - 1023;
-    if (e < -120 || e > 120) return div_ieee(d, v);
-    const double y0 = f2d_normal(__frcp_rn(f32_trunc(v)));   // |1 / v| in (2^-121, 2^120]: normal
+    unsigned lo, hi;
+    words(v, lo, hi);
+    if (hi_abs(hi) - 0x38700000u >= 0x0f100000u) return div_ieee(d, v);   // 2^-120 <= |v| < 2^121
+    const double y0 = f2d_normal(__frcp_rn(trunc_normal(lo, hi)));   // |1 / v| in (2^-121, 2^120]: normal
     const double e0 = fma(-v, y0, 1.0);
     const double y1 = fma(y0, fma(e0, e0, e0), y0);
     return d * y1;
@@ -217,11 +270,13 @@ __device__ __forceinline__ double f64_div(double d, double v)
 __device__ __forceinline__ double log1p_series(double r)
 {
     const double r2 = r * r;
-    const float rf = f32_trunc(r);
+    unsigned lo, hi;
+    words(r, lo, hi);
+    const float rf = trunc_small(lo, hi);
     float pf = __fmaf_rn(-0x1.0p-3f, rf, 0x1.24924ap-3f);   // -1/8, 1/7
     pf = __fmaf_rn(pf, rf, -0x1.555556p-3f);                // -1/6
     pf = __fmaf_rn(pf, rf, 0x1.99999ap-3f);                 // 1/5
-    double q = fma(r, f2d_normal(pf), -0.25);   // pf near 1/5: normal
+    double q = fma(r, f2d_normal_pos(pf), -0.25);   // pf near 1/5: normal
     q = fma(q, r, 1.0 / 3.0);
     q = fma(q, r, -0.5);
     return fma(r2, q, r);
@@ -245,8 +300,9 @@ static __device__ __noinline__ double log1p_far(double x, double u, double m, in
     return fma(de, ln2_hi, t0.y) + (fma(c, ru, lg) + fma(de, ln2_lo, Ll));
 }
 
-__device__ __forceinline__ double series_log1p(double x)
+static __device__ __noinline__ double series_log1p(double x)
 {
+    asm volatile("");
     const double u = 1.0 + x;
     const long long ub = bits(u);
     const bool ok = ub > 0LL && ub < 0x7ff0000000000000LL;   // 0 < u < inf
@@ -273,14 +329,53 @@ __device__ __forceinline__ double series_log1p(double x)
     return __longlong_as_double(ok ? bits(res) : special);   // -inf, +inf, NaN
 }
 
+// The row of f64_log_e_tab for u = 1 + x from the words of u: the exponent
+// and the top 8 fraction bits run through the rows of one exponent in order,
+// 256 of them, and each exponent has 257 (the bucket holding sqrt2 is split),
+// so the row is their sum plus one from sqrt2 on.  Rows outside the table (u
+// outside [2^-2 / sqrt2, 2^3 sqrt2), zero, infinite, NaN) come out of range.
+__device__ __forceinline__ unsigned log_row_f64(double u)
+{
+    unsigned lo, hi;
+    words(u, lo, hi);
+    const unsigned mh = hi & 0xfffffu;   // sqrt2's fraction: 0x6a09e 667f3bcd
+    const unsigned up = (mh > 0x6a09eu || (mh == 0x6a09eu && lo >= 0x667f3bcdu)) ? 1u : 0u;
+    return (hi >> 12) + (hi >> 20) + up - 262247u;
+}
+
+// log1p as series_log1p gives it, bit for bit.  Of u = 1 + x only the row is
+// needed, so it is taken from u in FP32 (x truncated: within 5 ulp of the
+// double's value wherever the row is in the table) except within 8 ulp of a
+// row's edge, where the FP64 sum decides (one lane in two thousand; the
+// branch is cheaper than that sum on every lane, the FP64 pipe being the
+// binding unit).
+__device__ __forceinline__ double fast_log1p(double x)
+{
+    unsigned lo, hi;
+    words(x, lo, hi);
+    // (|x| held below 2^126, whose rows are out of the table as well)
+    hi = min(hi_abs(hi), 0x47d00000u) | (hi & 0x80000000u);
+    const unsigned ub = __float_as_uint(1.0f + trunc_small(lo, hi));
+    const unsigned mf = ub & 0x7fffffu;
+    unsigned row = (ub >> 15) + (ub >> 23) + (mf >= 0x3504f3u ? 1u : 0u) - 31975u;
+    if (((ub + 8u) & 0x7fffu) < 16u || mf - (0x3504f3u - 8u) < 16u) row = log_row_f64(1.0 + x);
+    if (row >= (unsigned)(F64_LOG_NE * F64_LOG_N)) return series_log1p(x);
+    // (e ln2_hi + Lh, RN(e ln2_lo + Ll)), (R 2^-e, R 2^-e - 1)
+    const double2* t = reinterpret_cast<const double2*>(f64_log_e_tab) + 2 * row;
+    const double2 hl = __ldg(t), rp = __ldg(t + 1);
+    return hl.x + (log1p_series(fma(x, rp.x, rp.y)) + hl.y);
+}
+
 // e^r - 1 by its series to r^5 (the next term is below 1.5e-17 of the
 // result); the factor of r^4, 1/24 + r/120, in FP32: scaled by r^4 (below
 // 1.7e-10 of the result) its FP32 error stays below 0.1 ulp
 __device__ __forceinline__ double expm1_series(double r)
 {
     const double r2 = r * r;
-    const float pf = __fmaf_rn(0x1.111112p-7f, f32_trunc(r), 0x1.555556p-5f);   // 1/120, 1/24
-    double p = fma(f2d_normal(pf), r, 1.0 / 6.0);   // pf near 1/24: normal
+    unsigned lo, hi;
+    words(r, lo, hi);
+    const float pf = __fmaf_rn(0x1.111112p-7f, trunc_small(lo, hi), 0x1.555556p-5f);   // 1/120, 1/24
+    double p = fma(f2d_normal_pos(pf), r, 1.0 / 6.0);   // pf near 1/24: normal
     p = fma(p, r, 1.0 / 2.0);
     return fma(r2, p, r);
 }
@@ -326,25 +421,26 @@ __device__ __forceinline__ double series_expm1(double w)
     return expm1_far(r, dk, j, m);
 }
 
-// Exit time along one axis from the distance d to the reachable face
-// (face = +1, -1, or 0 when no face is reachable: +inf).  Written without
-// branches around the quotient and log1p so that the lanes of a warp stay
-// converged; lanes with no reachable face compute on harmless operands and
-// select +inf.  The values equal those of the branchy form (t1 = d / vp by
-// f64_div, z = A t1, t1 when z == 0 else log1p(z) * (1 / A)).
-__device__ __forceinline__ double f64_exit_time_d(double A, double iA, double d, double vp, int face)
+// Exit time along one axis from the distance d to its reachable face at the
+// particle velocity vp: t1 = d / vp by f64_div, z = A t1, t1 when z == 0,
+// else log1p(z) * (1 / A).
+__device__ __forceinline__ double f64_exit_time_d(double A, double iA, double d, double vp)
 {
-    const double t1 = f64_div(d, face ? vp : 1.0);
+    const double t1 = f64_div(d, vp);
     const double z = A * t1;
-    const bool lin = eq0(z) || !face;
-    const double te = lin ? t1 : series_log1p(lin ? 0.5 : z) * iA;
-    return face ? te : CUDART_INF;
+    const double te = fast_log1p(z) * iA;
+    unsigned lo, hi;
+    words(z, lo, hi);
+    return zero_w(lo, hi) ? t1 : te;
 }
 
-// the reachable face (v2pos / v1neg: the signs of the face velocities)
-__device__ __forceinline__ int f64_face(double vp, bool v2pos, bool v1neg)
+// the reachable face (+1, -1, 0: none) from the words of vp and the signs of
+// the face velocities (bits 1 and 2 of sg: v1 < 0, v2 > 0)
+__device__ __forceinline__ int f64_face(unsigned vlo, unsigned vhi, unsigned sg)
 {
-    return (gt0(vp) && v2pos) ? 1 : ((lt0(vp) && v1neg) ? -1 : 0);
+    const bool down = (int)vhi < 0;
+    const bool open = (sg & (down ? 2u : 4u)) != 0u && !zero_w(vlo, vhi);
+    return open ? (down ? -1 : 1) : 0;
 }
 
 // the signed distance to that face (D - pp up, -pp down and otherwise)
@@ -353,23 +449,16 @@ __device__ __forceinline__ double f64_face_dist(int face, double D, double pp)
     return face > 0 ? D - pp : neg(pp);
 }
 
-__device__ __forceinline__ double f64_exit_time(double A, double iA, double D, double vp, double pp, bool v2pos,
-                                                bool v1neg, int& face)
-{
-    face = f64_face(vp, v2pos, v1neg);
-    return f64_exit_time_d(A, iA, f64_face_dist(face, D, pp), vp, face);
-}
-
 // particle velocity at offset pp from face 1: v1 + A pp, one rounding
 __device__ __forceinline__ double f64_vel(double v1, double A, double pp) { return fma(A, pp, v1); }
 
-// analytic motion along one axis for a time dt, clamped to the cell
-// (the same values as: vp == 0 or dt == 0 -> pp; w == 0 -> pp + vp dt in one fma;
-// else pp + (vp * expm1(w)) * (1 / A), the last product and sum in one
-// fma); the operands are selected, so every lane issues one product and
-// one fma
-__device__ __forceinline__ double f64_move(double A, double iA, double D, double vp, double pp, double dt)
+// analytic motion along one axis for a time dt, clamped to the cell (vp == 0
+// or dt == 0 -> pp; w = A dt == 0 -> pp + vp dt in one fma; else pp +
+// (vp * expm1(w)) * (1 / A), the last product and sum in one fma): the form
+// for every w, out of line
+static __device__ __noinline__ double f64_move(double A, double iA, double D, double vp, double pp, double dt)
 {
+    asm volatile("");
     const bool still = eq0(vp) || eq0(dt);
     const double w = A * dt;
     const bool lin = eq0(w);
@@ -381,51 +470,112 @@ __device__ __forceinline__ double f64_move(double A, double iA, double D, double
     return still ? pp : pn;
 }
 
-// FP32 estimate of an exit time from an FP32 distance d and the FP64
-// particle velocity vp.  Relative error: the truncating conversions and
-// the approximate division give ~6e-7 on t1 = d / vp and on z = A t1, and
-// d from f32_face_dist below 6.2e-5; g(z) = ln(1 + z) / z is its series
-// for |z| < 2^-7, else __logf (absolute error at most 2^-21.41 on [1/2, 2],
-// 3 ulp outside) of u = fl(1 + z) over u - 1, in which the rounding of
-// 1 + z cancels (Goldberg 1991), or for z < -1/2 of the velocity ratio
-// u_exit / vp over z (the ratio, not 1 + z, carries the information
-// there): below 4.6e-5, since |ln u| >= 0.0078 wherever __logf is used.  In
-// all below 1.2e-4, a quarter of the 2^-11 that the candidate margin of
-// 2^-10 allows.  Velocities outside [1e-30, 1e30] (FP32
-// could not hold the quotients, and __fdividef gives 0 for divisors
-// beyond 2^126) or a NaN mark the estimate as untrusted.
-__device__ __forceinline__ float f32_estimate_f(int face, float d, double vp, float fA, float fue, bool& unsafe)
+// f64_move for |w| < 1.37 (all but a few in a thousand motions) and a result
+// inside the cell, without a branch, so that the motions of the axes of one
+// step interleave; `again` is set where f64_move has to give the result: w
+// outside (the tables' rows end at 2 ln2), or a result that is clamped.
+__device__ __forceinline__ double f64_move_fast(double A, double iA, double D, double vp, double pp, double dt,
+                                                bool& again)
 {
-    const float vf = f32_trunc(vp);
-    const float vs = face ? vf : 1.0f;
-    const float t1 = __fdividef(d, vs);
+    const double ln2_hi = 6.93147180369123816490e-01;
+    const double w = A * dt;
+    unsigned lo, hi;
+    words(w, lo, hi);
+    const bool lin = zero_w(lo, hi);
+    const bool out = hi_abs(hi) >= 0x3ff61000u;   // |w| >= 1.3789
+    const float sh = __fadd_rn(__fmul_rn(trunc_small(lo, hi), 0x1.715476p+8f), 12582912.0f);
+    const unsigned row = out ? 0u : __float_as_uint(sh) - 0x4b400000u - (unsigned)(F64_EXP_M0 * F64_EXP_N);
+    // (double)k for |k| <= 512: the FP32 integer's top bits, 0 for k = 0
+    const unsigned kb = __float_as_uint(__fadd_rn(sh, -12582912.0f));
+    const double dk = __hiloint2double(
+        kb == 0u ? 0 : (int)((((unsigned)((int)kb >> 3)) & 0x8fffffffu) + 0x38000000u), 0);
+    const double2 ab = __ldg(reinterpret_cast<const double2*>(f64_exp_ab_tab) + row);
+    const double r = fma(dk, -(ln2_hi / 256.0), w);
+    const double vem = vp * fma(ab.x, expm1_series(r), ab.y);
+    const double pn = fma(lin ? vp : vem, lin ? dt : iA, pp);
+    unsigned vlo, vhi, tlo, thi;
+    words(vp, vlo, vhi);
+    words(dt, tlo, thi);
+    const bool still = zero_w(vlo, vhi) || zero_w(tlo, thi);
+    // outside [0, D] as unsigned numbers (a set sign is the largest)
+    again = !still && (out || (unsigned long long)bits(pn) > (unsigned long long)bits(D));
+    return still ? pp : pn;
+}
+
+// FP32 estimate of an exit time from an FP32 distance d and the truncated
+// particle velocity vf.  Relative error: the truncation, the approximate
+// reciprocal (1 ulp) and the products give below 1e-6 on t1 = d / vf and on
+// z = A t1, and d from f32_face_dist below 6.2e-5; g(z) = ln(1 + z) / z is
+// its series for |z| < 2^-7, else the hardware base-2 logarithm (absolute
+// error at most 2^-22 on [1/2, 2], 1 ulp-scale outside) of u = fl(1 + z)
+// over u - 1, in which the rounding of 1 + z cancels (Goldberg 1991), or for
+// z < -1/2 of the velocity ratio u_exit / vp over z (the ratio, not 1 + z,
+// carries the information there): below 4.6e-5, since |ln u| >= 0.0078
+// wherever the logarithm is used.  In all below 1.2e-4, a quarter of the
+// 2^-11 that the candidate margin of 2^-10 allows.
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float lg2_approx(float x)
+{
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float f32_estimate(float d, float vf, float fA, float fue)
+{
+    const float iv = rcp_approx(vf);
+    const float t1 = d * iv;
     const float z = fA * t1;
     // both forms, selected (no divergent branch)
     const bool near_m1 = z < -0.5f;
     const float u = 1.0f + z;
-    const float L = __logf(near_m1 ? __fdividef(fue, vs) : u);
-    const float gl = __fdividef(L, near_m1 ? z : u - 1.0f);
-    const float gs = 1.0f + z * (-0.5f + z * (1.0f / 3.0f + z * (-0.25f + z * 0.2f)));
-    const float g = fabsf(z) < 0.0078125f ? gs : gl;
-    const float e = t1 * g;
-    unsafe = face != 0 && (!(fabsf(vf) >= 1e-30f) || !(fabsf(vf) <= 1e30f) || !(e == e));
-    return face ? e : CUDART_INF_F;
+    const float L = lg2_approx(near_m1 ? fue * iv : u) * 0.693147181f;
+    const float gl = L * rcp_approx(near_m1 ? z : u - 1.0f);
+    const float gs = __fmaf_rn(z, __fmaf_rn(z, __fmaf_rn(z, __fmaf_rn(z, 0.2f, -0.25f), 1.0f / 3.0f), -0.5f), 1.0f);
+    return t1 * (fabsf(z) < 0.0078125f ? gs : gl);
 }
+
+// velocities whose estimates are trusted: |vp| in [2^-100, 2^100) (FP32
+// could not hold the quotients of others), from the high word
+__device__ __forceinline__ bool vel_trusted(unsigned vhi) { return hi_abs(vhi) - 0x39b00000u < 0x0c800000u; }
 
 // FP32 distance to the reachable face for the estimates without an FP64
 // subtraction: -pp truncated, or D - pp from the truncated operands (error
 // below 2^-23 D plus one FP32 rounding, so below 6.2e-5 relative while the
-// distance is at least 2^-9 D); nearer the face (rare) the truncated FP64
-// difference, out of line
-static __device__ __noinline__ float f32_dist_near(double D, double pp) { return f32_trunc(D - pp); }
-
-__device__ __forceinline__ float f32_face_dist(int face, double D, double pp)
+// distance is at least 2^-9 D); nearer the face (close is set; rare) the
+// caller takes the truncated FP64 difference
+__device__ __forceinline__ float f32_face_dist(int face, float Df, double pp, bool& close)
 {
-    const float pf = f32_trunc(pp);
-    if (face <= 0) return -pf;
-    const float Df = f32_trunc(D);
-    const float d = Df - pf;
-    return d >= Df * 0x1.0p-9f ? d : f32_dist_near(D, pp);
+    unsigned lo, hi;
+    words(pp, lo, hi);
+    const float pf = trunc_pos(lo, hi);
+    const float up = Df - pf;
+    close = face > 0 && up < Df * 0x1.0p-9f;
+    return face > 0 ? up : -pf;
+}
+
+// The exit axis's screening: axes whose exact exit time has to be formed.
+// e: the estimates of the reachable axes (reach: bit a), infinity for the
+// others; doubt: some reachable axis's estimate cannot be trusted.  Gives
+// the leading axis (-1: none reachable) and the others that may still win:
+// those within 2^-10 of it (the estimates are within 1.2e-4 of the exact
+// times), or every reachable one when in doubt or nothing is finite.
+__device__ __forceinline__ int screen(float e0, float e1, float e2, unsigned reach, bool doubt, unsigned& rest)
+{
+    const float em = fminf(fminf(e0, e1), e2);
+    const float thr = em * (1.0f + 0.0009765625f);
+    int a0 = e0 == em ? 0 : (e1 == em ? 1 : 2);
+    rest = (e0 <= thr ? 1u : 0u) | (e1 <= thr ? 2u : 0u) | (e2 <= thr ? 4u : 0u);
+    if (doubt || !(em < CUDART_INF_F)) {
+        a0 = __ffs(reach) - 1;
+        rest = reach;
+    }
+    rest &= ~(1u << (a0 & 31));
+    return a0;
 }
 
 }  // namespace mp

@@ -45,14 +45,37 @@ struct __align__(32) CellF32 {
 };
 static_assert(sizeof(CellF32) == 32, "CellF32 is one 32-byte sector");
 
+// a column's, row's or layer's size, with its FP32 truncation for the
+// FP64 path's screening
+struct __align__(16) AxisCell {
+    double D;
+    float f;
+    float pad;
+};
+
+// x truncated toward zero to FP32 (below the normal range 0, above infinity);
+// x > 0
+inline float host_f32_trunc(double x)
+{
+    if (x < 1.17549435082228751e-38) return 0.0f;
+    float f = (float)x;
+    if ((double)f > x) f = __builtin_nextafterf(f, 0.0f);
+    return x >= 3.4028236692093846e+38 ? __builtin_inff() : f;
+}
+
+// cell sizes above this are beyond the FP32 screening (2^120 m)
+constexpr double SCREEN_MAX_D = 1.329227995784916e+36;
+
 struct DevField {
     int nlay, nrow, ncol;
+    int no_screen;     // some cell size is above SCREEN_MAX_D: every reachable axis is evaluated exactly
     long long ncell;
     const CellF64* rec64;
     const CellF32* rec32;
     const double* delr;
     const double* delc;
     const double* dz;
+    const AxisCell* ax;   // sizes of the columns, then the rows, then the layers
     const double* xf;  // [ncol+1]
     const double* yf;  // [nrow+1]
     const double* zf;  // [nlay+1]
@@ -219,6 +242,7 @@ struct __align__(16) UsgSub {
 };
 
 struct DevUsg {
+    int no_screen;            // as DevField's
     long long ncell;
     long long nsub;
     const UsgCell* cell;

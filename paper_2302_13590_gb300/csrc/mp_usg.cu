@@ -164,7 +164,8 @@ struct UsgEngine {
         int st;
         int ef;
         int in_sink;
-        double tev;
+        unsigned cap;     // as in the rectilinear engine
+        long long tev;
     };
 
     __device__ __forceinline__ double gx(const State& s) const { return __ldg(&u.geo[s.c].o[0]) + s.x0; }
@@ -186,11 +187,11 @@ struct UsgEngine {
         z = ok ? gz(s) : CUDART_NAN;
     }
 
-    __device__ __forceinline__ double next_event(const State& s) const
+    __device__ __forceinline__ long long next_event(const State& s) const
     {
         const Req& R = b.reqs[s.r];
         const double tk = s.kn < R.p.n_times ? __ldg(R.o.times + s.kn) : CUDART_INF;
-        return fmin(tk, R.p.t_stop);
+        return bound_key(ge_d(tk, R.p.t_stop) ? R.p.t_stop : tk);
     }
 
     template <bool TS>
@@ -210,6 +211,7 @@ struct UsgEngine {
         s.x0 = in.px[q]; s.x1 = in.py[q]; s.x2 = in.pz[q];
         s.t = in.t[q];
         s.steps = in.steps ? in.steps[q] : 0u;
+        s.cap = p.max_steps > 0xffffffffLL ? 0xffffffffu : (unsigned)p.max_steps;
         s.h = FNV_INIT;
         s.kn = 0;
         s.ef = (s.steps && in.exit_face) ? (int)in.exit_face[q] : MP_FACE_NONE;
@@ -238,7 +240,7 @@ struct UsgEngine {
             }
         }
         if (s.st == MP_ST_ACTIVE && s.t >= p.t_stop) s.st = MP_ST_TIME;
-        s.tev = TS ? next_event(s) : p.t_stop;
+        s.tev = TS ? next_event(s) : bound_key(p.t_stop);
     }
 
     struct RecQ {
@@ -265,12 +267,19 @@ struct UsgEngine {
         const UsgCell& k = u.cell[c];
         const UsgGeo& g = u.geo[c];
         const double p0 = Q.p0[slot], p1 = Q.p1[slot], p2 = Q.p2[slot], tau = Q.tau[slot];
-        const double x = __ldg(&g.o[0]) + f64_move(__ldg(&k.Ax), __ldg(&k.iAx), __ldg(&g.D[0]),
-                                                   f64_vel(__ldg(&k.v1x), __ldg(&k.Ax), p0), p0, tau);
-        const double y = __ldg(&g.o[1]) + f64_move(__ldg(&k.Ay), __ldg(&k.iAy), __ldg(&g.D[1]),
-                                                   f64_vel(__ldg(&k.v1y), __ldg(&k.Ay), p1), p1, tau);
-        const double z = __ldg(&g.o[2]) + f64_move(__ldg(&k.Az), __ldg(&k.iAz), __ldg(&g.D[2]),
-                                                   f64_vel(__ldg(&k.v1z), __ldg(&k.Az), p2), p2, tau);
+        const double Ax = __ldg(&k.Ax), Ay = __ldg(&k.Ay), Az = __ldg(&k.Az);
+        const double iAx = __ldg(&k.iAx), iAy = __ldg(&k.iAy), iAz = __ldg(&k.iAz);
+        const double D0 = __ldg(&g.D[0]), D1 = __ldg(&g.D[1]), D2 = __ldg(&g.D[2]);
+        const double vx = f64_vel(__ldg(&k.v1x), Ax, p0), vy = f64_vel(__ldg(&k.v1y), Ay, p1),
+                     vz = f64_vel(__ldg(&k.v1z), Az, p2);
+        bool again;
+        double nx = f64_move_fast(Ax, iAx, D0, vx, p0, tau, again);
+        if (again) nx = f64_move(Ax, iAx, D0, vx, p0, tau);
+        double ny = f64_move_fast(Ay, iAy, D1, vy, p1, tau, again);
+        if (again) ny = f64_move(Ay, iAy, D1, vy, p1, tau);
+        double nz = f64_move_fast(Az, iAz, D2, vz, p2, tau, again);
+        if (again) nz = f64_move(Az, iAz, D2, vz, p2, tau);
+        const double x = __ldg(&g.o[0]) + nx, y = __ldg(&g.o[1]) + ny, z = __ldg(&g.o[2]) + nz;
         store_record(R.o.ts + (long long)Q.kk[slot] * R.p.n + Q.q[slot], x, y, z, c, Q.st[slot]);
     }
 
@@ -366,9 +375,9 @@ struct UsgEngine {
         double vp[3] = {0, 0, 0}, tmin = 0, t_end = 0;
         int fc[3] = {0, 0, 0}, ax = -1;
         if (live) {
-            if ((long long)s.steps >= p.max_steps) {
+            if (s.steps >= s.cap && (long long)s.steps >= p.max_steps) {
                 s.st = MP_ST_STEP_CAP;
-            } else if ((unsigned long long)s.c >= (unsigned long long)u.ncell) {
+            } else if ((unsigned)s.c >= (unsigned)u.ncell) {
                 atomicCAS(o.counters + COUNTER_ERR, 0ULL, (unsigned long long)q + 1ULL);
                 s.st = MP_ST_INVALID_RELEASE;
             } else {
@@ -381,65 +390,63 @@ struct UsgEngine {
                 const double2 q0 = __ldg(gp + 0), q1 = __ldg(gp + 1), q2 = __ldg(gp + 2);
                 v1[0] = r0.x; A[0] = r0.y; iA[0] = r1.x; v1[1] = r1.y; A[1] = r2.x; iA[1] = r2.y;
                 v1[2] = r3.x; A[2] = r3.y; iA[2] = r4.x;
-                const unsigned long long sg = (unsigned long long)__double_as_longlong(r4.y);
+                const unsigned sg = (unsigned)__double_as_longlong(r4.y);   // (12 bits are in use)
                 org[0] = q0.x; org[1] = q0.y; org[2] = q1.x; D[0] = q1.y; D[1] = q2.x; D[2] = q2.y;
                 const double pp[3] = {s.x0, s.x1, s.x2};
-                bool p2[3], n1[3];
-                float dd[3];
+                // the screening of the exit axis and the exact times of its
+                // candidates, as in the rectilinear engine
+                float dd[3], te3[3];
+                bool close[3], doubt = u.no_screen;
+                unsigned reach = 0u, vlo[3], vhi[3];
                 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     vp[a] = f64_vel(v1[a], A[a], pp[a]);
-                    p2[a] = (sg >> (4 * a + 2)) & 1ULL;
-                    n1[a] = (sg >> (4 * a + 1)) & 1ULL;
-                    fc[a] = f64_face(vp[a], p2[a], n1[a]);
-                    dd[a] = f32_face_dist(fc[a], D[a], pp[a]);
+                    words(vp[a], vlo[a], vhi[a]);
+                    fc[a] = f64_face(vlo[a], vhi[a], sg >> (4 * a));
+                    unsigned lo, hi;
+                    words(D[a], lo, hi);
+                    dd[a] = f32_face_dist(fc[a], trunc_pos(lo, hi), pp[a], close[a]);
+                    reach |= fc[a] ? 1u << a : 0u;
                 }
-                // FP32 estimates of the three exit times (from FP32 face
-                // distances); the exact FP64 time of the leading one, and of
-                // every axis within 2^-10 of it or with an untrusted
-                // estimate (the same exit axis and time as evaluating all
-                // three exactly)
-                bool u0, u1, u2;
-                const float e0 = f32_estimate_f(fc[0], dd[0], vp[0], g0.z,
-                                                fc[0] > 0 ? g0.y : g0.x, u0);
-                const float e1 = f32_estimate_f(fc[1], dd[1], vp[1], g1.y,
-                                                fc[1] > 0 ? g1.x : g0.w, u1);
-                const float e2 = f32_estimate_f(fc[2], dd[2], vp[2], g2.x,
-                                                fc[2] > 0 ? g1.w : g1.z, u2);
-                float em = CUDART_INF_F;
-                int a0 = -1;
-                if (fc[0] && !u0 && e0 < em) { em = e0; a0 = 0; }
-                if (fc[1] && !u1 && e1 < em) { em = e1; a0 = 1; }
-                if (fc[2] && !u2 && e2 < em) { em = e2; a0 = 2; }
-                const float thr = em * (1.0f + 0.0009765625f);
-                const unsigned cand = ((fc[0] && (u0 || e0 <= thr)) ? 1u : 0u) | ((fc[1] && (u1 || e1 <= thr)) ? 2u : 0u) |
-                                      ((fc[2] && (u2 || e2 <= thr)) ? 4u : 0u);
-                if (a0 < 0 && cand) a0 = __ffs(cand) - 1;
+                if (close[0] || close[1] || close[2]) {
+                    #pragma unroll
+                    for (int a = 0; a < 3; ++a)
+                        if (close[a]) dd[a] = f32_trunc(D[a] - pp[a]);
+                }
+                const float fA[3] = {g0.z, g1.y, g2.x};
+                const float fu[3] = {fc[0] > 0 ? g0.y : g0.x, fc[1] > 0 ? g1.x : g0.w, fc[2] > 0 ? g1.w : g1.z};
+                #pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    const float t = f32_estimate(dd[a], trunc_normal(vlo[a], vhi[a]), fA[a], fu[a]);
+                    doubt = doubt || (fc[a] && !(vel_trusted(vhi[a]) && t < CUDART_INF_F));
+                    te3[a] = fc[a] ? t : CUDART_INF_F;
+                }
+                unsigned rest;
+                const int a0 = screen(te3[0], te3[1], te3[2], reach, doubt, rest);
                 tmin = CUDART_INF;
                 if (a0 >= 0) {
-                    const int fa0 = sel3(a0, fc[0], fc[1], fc[2]);
                     const double te = f64_exit_time_d(
                         sel3(a0, A[0], A[1], A[2]), sel3(a0, iA[0], iA[1], iA[2]),
-                        f64_face_dist(fa0, sel3(a0, D[0], D[1], D[2]), sel3(a0, pp[0], pp[1], pp[2])),
-                        sel3(a0, vp[0], vp[1], vp[2]), fa0);
+                        f64_face_dist(sel3(a0, fc[0], fc[1], fc[2]), sel3(a0, D[0], D[1], D[2]),
+                                      sel3(a0, pp[0], pp[1], pp[2])),
+                        sel3(a0, vp[0], vp[1], vp[2]));
                     // the other candidates (every reachable axis when the
                     // leading time is unusable): smallest wins, ties to the
                     // lower axis
-                    unsigned rest = cand & ~(1u << a0);
-                    if (lt_inf(te)) {
+                    if (is_finite(te)) {
                         tmin = te;
                         ax = a0;
                     } else {
-                        rest = ((fc[0] ? 1u : 0u) | (fc[1] ? 2u : 0u) | (fc[2] ? 4u : 0u)) & ~(1u << a0);
+                        rest = reach & ~(1u << a0);
                     }
                     while (rest) {
                         const int a = __ffs(rest) - 1;
                         rest &= rest - 1;
-                        const int fa = sel3(a, fc[0], fc[1], fc[2]);
                         const double t = f64_exit_time_d(
                             sel3(a, A[0], A[1], A[2]), sel3(a, iA[0], iA[1], iA[2]),
-                            f64_face_dist(fa, sel3(a, D[0], D[1], D[2]), sel3(a, pp[0], pp[1], pp[2])),
-                            sel3(a, vp[0], vp[1], vp[2]), fa);
+                            f64_face_dist(sel3(a, fc[0], fc[1], fc[2]), sel3(a, D[0], D[1], D[2]),
+                                          sel3(a, pp[0], pp[1], pp[2])),
+                            sel3(a, vp[0], vp[1], vp[2]));
                         if (t < tmin || (t == tmin && a < ax)) {
                             tmin = t;
                             ax = a;
@@ -448,15 +455,17 @@ struct UsgEngine {
                 }
                 s.steps++;
                 t_end = s.t + tmin;
-                if (ax < 0 && s.in_sink) path = P_CAPTURE;
-                else if (ax < 0 && !(p.t_stop < CUDART_INF)) path = P_NOEXIT;
-                else if (ax < 0 || ge_d(t_end, p.t_stop)) path = P_TIME;
-                else path = P_CROSS;
-                if (TS && path != P_CAPTURE && (ax < 0 || ge_d(t_end, s.tev))) {
-                    const double t_rec = path == P_NOEXIT ? CUDART_INF : (path == P_TIME ? p.t_stop : t_end);
-                    int kk = s.kn;
-                    while (kk < p.n_times && __ldg(o.times + kk) <= t_rec) kk++;
-                    m = kk - s.kn;
+                path = P_CROSS;
+                if (ax < 0 || tkey(t_end) >= s.tev) {   // (the stop time is never before tev)
+                    if (ax < 0 && s.in_sink) path = P_CAPTURE;
+                    else if (ax < 0 && !(p.t_stop < CUDART_INF)) path = P_NOEXIT;
+                    else if (ax < 0 || ge_d(t_end, p.t_stop)) path = P_TIME;
+                    if (TS && path != P_CAPTURE) {
+                        const double t_rec = path == P_NOEXIT ? CUDART_INF : (path == P_TIME ? p.t_stop : t_end);
+                        int kk = s.kn;
+                        while (kk < p.n_times && ge_d(t_rec, __ldg(o.times + kk))) kk++;
+                        m = kk - s.kn;
+                    }
                 }
             }
         }
@@ -490,12 +499,18 @@ struct UsgEngine {
         // axis is put on its face
         const double dt = tmin;
         const int a1 = ax == 0 ? 1 : 0, a2 = ax == 2 ? 1 : 2;
-        const double n1v = f64_move(sel3(a1, A[0], A[1], A[2]), sel3(a1, iA[0], iA[1], iA[2]),
-                                    sel3(a1, D[0], D[1], D[2]), sel3(a1, vp[0], vp[1], vp[2]),
-                                    sel3(a1, pp[0], pp[1], pp[2]), dt);
-        const double n2v = f64_move(sel3(a2, A[0], A[1], A[2]), sel3(a2, iA[0], iA[1], iA[2]),
-                                    sel3(a2, D[0], D[1], D[2]), sel3(a2, vp[0], vp[1], vp[2]),
-                                    sel3(a2, pp[0], pp[1], pp[2]), dt);
+        const double B1 = sel3(a1, A[0], A[1], A[2]), iB1 = sel3(a1, iA[0], iA[1], iA[2]);
+        const double B2 = sel3(a2, A[0], A[1], A[2]), iB2 = sel3(a2, iA[0], iA[1], iA[2]);
+        const double E1 = sel3(a1, D[0], D[1], D[2]), E2 = sel3(a2, D[0], D[1], D[2]);
+        const double w1 = sel3(a1, vp[0], vp[1], vp[2]), w2 = sel3(a2, vp[0], vp[1], vp[2]);
+        const double y1 = sel3(a1, pp[0], pp[1], pp[2]), y2 = sel3(a2, pp[0], pp[1], pp[2]);
+        bool again1, again2;
+        double n1v = f64_move_fast(B1, iB1, E1, w1, y1, dt, again1);
+        double n2v = f64_move_fast(B2, iB2, E2, w2, y2, dt, again2);
+        if (again1 || again2) {
+            if (again1) n1v = f64_move(B1, iB1, E1, w1, y1, dt);
+            if (again2) n2v = f64_move(B2, iB2, E2, w2, y2, dt);
+        }
         const int side = sel3(ax, fc[0], fc[1], fc[2]);
         const double pf = side > 0 ? sel3(ax, D[0], D[1], D[2]) : 0.0;
         pp[0] = ax == 0 ? pf : n1v;
