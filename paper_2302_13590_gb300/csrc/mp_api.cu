@@ -129,6 +129,7 @@ struct Request {
     DevOut d{};
     void* buf = nullptr;
     size_t bytes = 0;
+    unsigned long long* queue = nullptr;   // queue head of its own launches, in buf after the counters
     cudaStream_t stream = nullptr;
     cudaEvent_t k0 = nullptr, k1 = nullptr;
     bool graph_owned = false;   // outputs of a captured graph: freed with it, events shared
@@ -638,12 +639,8 @@ int mp_release_group(mp_ctx* ctx, const mp_field* f, const mp_release_desc* r, v
         delete g;
         return fail(MP_ERR_INVALID_ARG, "mp_release_group: box releases need a rectilinear grid");
     }
-    cudaError_t e = cudaMemsetAsync(g->d.steps, 0, 4 * (size_t)n, s);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(buf, s);
-        delete g;
-        return cuda_fail(e, "mp_release_group");
-    }
+    // (the release kernels write the zero step counts)
+    cudaError_t e = cudaSuccess;
     if (r->kind == MP_RELEASE_BOX) {
         e = launch_release_box(f->d, g->d, n, r->lo, r->hi, r->seed, r->id_offset, s);
     } else if (n > 0) {
@@ -754,9 +751,23 @@ int mp_track_launches(const mp_track_opts* o, int32_t* launches)
 
 namespace {
 
+// a request's output times as the device holds them: the FP64 times, then at
+// the next 256-byte boundary the same as FP32 pairs
+size_t times_bytes(int nt) { return align256(sizeof(double) * (size_t)nt) + sizeof(float2) * (size_t)nt; }
+
+void pack_times(const double* t, int nt, char* dst)
+{
+    memcpy(dst, t, sizeof(double) * (size_t)nt);
+    float2* ff = reinterpret_cast<float2*>(dst + align256(sizeof(double) * (size_t)nt));
+    for (int k = 0; k < nt; ++k) split_ff(t[k], ff[k].x, ff[k].y);
+}
+
 // Check options and allocate one request's outputs (stream-ordered); fills
-// the request's device descriptor on the host side.
-int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream_t s, Request** out,
+// the request's device descriptor on the host side.  own: the request is
+// launched by itself or replayed, so its output times go into its own buffer
+// (one copy) and its counters and queue word are zeroed here; otherwise the
+// launch's table carries the times and one kernel zeroes every counter.
+int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream_t s, bool own, Request** out,
                     mp::Req* hreq, unsigned* modes)
 {
     if (!g || !o) return fail(MP_ERR_INVALID_ARG, "mp_track: NULL argument");
@@ -818,7 +829,7 @@ int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream
     r->d.exit_face = reinterpret_cast<uint8_t*>(take((size_t)n));
     r->d.hash = reinterpret_cast<unsigned long long*>(take(8 * (size_t)n));
     r->d.counters = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * N_COUNTERS));
-    take(sizeof(unsigned long long));   // spare word (queue head of a single-request launch)
+    r->queue = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long)));
     r->d.ts = nullptr;
     r->d.times = nullptr;
     r->d.times_ff = nullptr;
@@ -835,15 +846,13 @@ int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream
         r->d.path = reinterpret_cast<mp_path_record*>(take(sizeof(mp_path_record) * (size_t)r->d.path_cap));
     }
     cudaError_t e = cudaSuccess;
-    if (nt > 0) e = cudaMemcpyAsync(const_cast<double*>(r->d.times), o->times, sizeof(double) * nt,
-                                    cudaMemcpyHostToDevice, s);
-    if (nt > 0 && e == cudaSuccess) {
-        std::vector<float2> ff((size_t)nt);
-        for (int k = 0; k < nt; ++k) split_ff(o->times[k], ff[k].x, ff[k].y);
-        e = cudaMemcpyAsync(const_cast<float2*>(r->d.times_ff), ff.data(), sizeof(float2) * nt,
-                            cudaMemcpyHostToDevice, s);
+    if (own && nt > 0) {
+        std::vector<char> h(times_bytes(nt));
+        pack_times(o->times, nt, h.data());
+        e = cudaMemcpyAsync(const_cast<double*>(r->d.times), h.data(), h.size(), cudaMemcpyHostToDevice, s);
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(r->d.counters, 0, sizeof(unsigned long long) * N_COUNTERS, s);
+    if (own && e == cudaSuccess)   // (the queue word follows the counters)
+        e = cudaMemsetAsync(r->d.counters, 0, align256(sizeof(unsigned long long) * N_COUNTERS) + sizeof(unsigned long long), s);
     if (e == cudaSuccess) e = cudaEventCreate(&r->k0);
     if (e == cudaSuccess) e = cudaEventCreate(&r->k1);
     if (e != cudaSuccess) {
@@ -888,32 +897,60 @@ void drop_request(Request* r)
 // "Multiprocessing": a single particle loop over every particle).
 // ev: 1 records the requests' start events before the launch, 2 their end
 // events after it (a request made of several launches records each once).
-int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, int n, int precision, int schedule,
-                    int block, int spf, unsigned modes, cudaStream_t s, unsigned ev = 3)
+// One request (prepared with own) needs no table: its descriptor travels as a
+// kernel parameter.  Several (prepared without) get one table in one copy:
+// descriptors, starts, a zero queue head and the output times, each distinct
+// times array once.
+int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, const mp_track_opts* const* opts, int n,
+                    int precision, int schedule, int block, int spf, unsigned modes, cudaStream_t s, unsigned ev = 3)
 {
-    size_t off = 0;
-    const size_t o_req = off; off = align256(off + sizeof(mp::Req) * (size_t)n);
-    const size_t o_st = off; off = align256(off + sizeof(long long) * ((size_t)n + 1));
-    const size_t o_q = off; off = align256(off + sizeof(unsigned long long));
-    char* tbl = nullptr;
-    if (cudaMallocAsync(&tbl, off, s) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(MP_ERR_OOM, "mp_track: device allocation failed");
-    }
-    std::vector<long long> starts((size_t)n + 1, 0);
-    for (int i = 0; i < n; ++i) starts[i + 1] = starts[i] + hreqs[i].p.n;
-    cudaError_t e = cudaMemcpyAsync(tbl + o_req, hreqs, sizeof(mp::Req) * (size_t)n, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(tbl + o_st, starts.data(), sizeof(long long) * ((size_t)n + 1), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tbl + o_q, 0, sizeof(unsigned long long), s);
-    for (int i = 0; i < n && e == cudaSuccess && (ev & 1u); ++i) e = cudaEventRecord(rs[i]->k0, s);
     mp::Batch b{};
-    b.reqs = reinterpret_cast<const mp::Req*>(tbl + o_req);
-    b.starts = reinterpret_cast<const long long*>(tbl + o_st);
     b.n_reqs = n;
-    b.n_total = starts[n];
     b.steps_per_fetch = spf > 0 ? spf : 4;
-    b.queue = reinterpret_cast<unsigned long long*>(tbl + o_q);
+    char* tbl = nullptr;
+    cudaError_t e = cudaSuccess;
+    if (n == 1) {
+        b.one = hreqs[0];
+        b.n_total = hreqs[0].p.n;
+        b.queue = rs[0]->queue;
+        if (!(ev & 1u)) e = cudaMemsetAsync(b.queue, 0, sizeof(unsigned long long), s);   // (a later launch of it)
+    } else {
+        size_t off = 0;
+        const size_t o_req = off; off = align256(off + sizeof(mp::Req) * (size_t)n);
+        const size_t o_st = off; off = align256(off + sizeof(long long) * ((size_t)n + 1));
+        const size_t o_q = off; off = align256(off + sizeof(unsigned long long));
+        std::vector<size_t> o_t((size_t)n, 0);
+        for (int i = 0; i < n; ++i) {
+            if (hreqs[i].p.n_times == 0) continue;
+            const bool again = i > 0 && opts[i]->times == opts[i - 1]->times &&
+                               hreqs[i].p.n_times == hreqs[i - 1].p.n_times;
+            o_t[i] = again ? o_t[i - 1] : off;
+            if (!again) off = align256(off + times_bytes(hreqs[i].p.n_times));
+        }
+        if (cudaMallocAsync(&tbl, off, s) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(MP_ERR_OOM, "mp_track: device allocation failed");
+        }
+        std::vector<char> h(off, 0);
+        mp::Req* hr = reinterpret_cast<mp::Req*>(h.data() + o_req);
+        long long* st = reinterpret_cast<long long*>(h.data() + o_st);
+        for (int i = 0; i < n; ++i) {
+            hr[i] = hreqs[i];
+            st[i + 1] = st[i] + hreqs[i].p.n;
+            const int nt = hreqs[i].p.n_times;
+            if (nt == 0) continue;
+            if (i == 0 || o_t[i] != o_t[i - 1]) pack_times(opts[i]->times, nt, h.data() + o_t[i]);
+            hr[i].o.times = reinterpret_cast<double*>(tbl + o_t[i]);
+            hr[i].o.times_ff = reinterpret_cast<float2*>(tbl + o_t[i] + align256(sizeof(double) * (size_t)nt));
+        }
+        e = cudaMemcpyAsync(tbl, h.data(), off, cudaMemcpyHostToDevice, s);
+        b.reqs = reinterpret_cast<const mp::Req*>(tbl + o_req);
+        b.starts = reinterpret_cast<const long long*>(tbl + o_st);
+        b.n_total = st[n];
+        b.queue = reinterpret_cast<unsigned long long*>(tbl + o_q);
+        if (e == cudaSuccess) e = launch_zero_counters(b, s);
+    }
+    for (int i = 0; i < n && e == cudaSuccess && (ev & 1u); ++i) e = cudaEventRecord(rs[i]->k0, s);
     const int blk = block > 0 ? block : 128;
     if (e == cudaSuccess) {
         const mp::DevField& fd = *mp::field_device_view(f);
@@ -924,7 +961,7 @@ int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, int n
         if (e == cudaSuccess) e = mp::launch_spread_window(b, s);
     }
     for (int i = 0; i < n && e == cudaSuccess && (ev & 2u); ++i) e = cudaEventRecord(rs[i]->k1, s);
-    cudaFreeAsync(tbl, s);
+    if (tbl) cudaFreeAsync(tbl, s);
     if (e != cudaSuccess) return cuda_fail(e, "mp_track: launch");
     return MP_OK;
 }
@@ -1005,9 +1042,13 @@ int mp_track_batch(mp_ctx* ctx, int n, mp_group* const* groups, const mp_track_o
     std::vector<Request*> rs((size_t)n, nullptr);
     std::vector<mp::Req> hr((size_t)n);
     std::vector<char> ts((size_t)n, 0);
+    int of_prec[3] = {0, 0, 0};
+    for (int i = 0; i < n; ++i)
+        if (opts[i].precision >= 0 && opts[i].precision < 3) of_prec[opts[i].precision]++;
     for (int i = 0; i < n; ++i) {
         unsigned md = 0;
-        const int rc = prepare_request(ctx, groups[i], &opts[i], s, &rs[i], &hr[i], &md);
+        const bool own = opts[i].precision >= 0 && opts[i].precision < 3 && of_prec[opts[i].precision] == 1;
+        const int rc = prepare_request(ctx, groups[i], &opts[i], s, own, &rs[i], &hr[i], &md);
         if (rc != MP_OK) {
             for (int k = 0; k < i; ++k) drop_request(rs[k]);
             return rc;
@@ -1018,6 +1059,7 @@ int mp_track_batch(mp_ctx* ctx, int n, mp_group* const* groups, const mp_track_o
     for (int prec = 0; prec < 3; ++prec) {
         std::vector<Request*> sel;
         std::vector<mp::Req> sreq;
+        std::vector<const mp_track_opts*> sopt;
         unsigned any_modes = 0;
         int first = -1;
         for (int i = 0; i < n; ++i)
@@ -1025,12 +1067,13 @@ int mp_track_batch(mp_ctx* ctx, int n, mp_group* const* groups, const mp_track_o
                 if (first < 0) first = i;
                 sel.push_back(rs[i]);
                 sreq.push_back(hr[i]);
+                sopt.push_back(&opts[i]);
                 any_modes |= (unsigned)ts[i];
             }
         if (sel.empty()) continue;
         int sched = 0, blk = 0, spf = 0;
         resolve_launch(ctx, groups[0]->field, prec, (any_modes & mp::MODE_TS) != 0, opts[first], &sched, &blk, &spf);
-        const int rc = launch_requests(groups[0]->field, sel.data(), sreq.data(), (int)sel.size(), prec,
+        const int rc = launch_requests(groups[0]->field, sel.data(), sreq.data(), sopt.data(), (int)sel.size(), prec,
                                        sched, blk, spf, any_modes, s);
         if (rc != MP_OK) {
             cudaStreamSynchronize(s);
@@ -1080,7 +1123,7 @@ int mp_track_periods(mp_ctx* ctx, mp_group* g, int n_periods, const mp_field* co
     Request* r = nullptr;
     mp::Req hr;
     unsigned modes = 0;
-    int rc = prepare_request(ctx, g, o, s, &r, &hr, &modes);
+    int rc = prepare_request(ctx, g, o, s, true, &r, &hr, &modes);
     if (rc != MP_OK) return rc;
     r->fields.assign(fields, fields + n_periods);
     // the periods advance a request-owned copy of the group's state
@@ -1109,7 +1152,7 @@ int mp_track_periods(mp_ctx* ctx, mp_group* g, int n_periods, const mp_field* co
         h.p.last = last ? 1 : 0;
         int sched = 0, blk = 0, spf = 0;
         resolve_launch(ctx, fields[p], o->precision, (modes & mp::MODE_TS) != 0, *o, &sched, &blk, &spf);
-        rc = launch_requests(fields[p], &r, &h, 1, o->precision, sched, blk, spf, modes, s,
+        rc = launch_requests(fields[p], &r, &h, &o, 1, o->precision, sched, blk, spf, modes, s,
                              (p == 0 ? 1u : 0u) | (last ? 2u : 0u));
         if (rc != MP_OK) {
             cudaStreamSynchronize(s);
@@ -1477,10 +1520,11 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
         const Cand c = ci == 0 ? cands[0] : cands[ci - 1];
         Request* r = nullptr;
         mp::Req hr;
-        int rc = prepare_request(ctx, g, &oo, s, &r, &hr, &modes);
+        int rc = prepare_request(ctx, g, &oo, s, true, &r, &hr, &modes);
         if (rc != MP_OK) return rc;
         if (sample > 0 && hr.p.n > sample) hr.p.n = sample;
-        rc = launch_requests(g->field, &r, &hr, 1, o->precision, c.sched, c.block, c.spf, modes, s);
+        const mp_track_opts* po = &oo;
+        rc = launch_requests(g->field, &r, &hr, &po, 1, o->precision, c.sched, c.block, c.spf, modes, s);
         if (rc == MP_OK) rc = wait_event(r->k1, -1);
         float ms = 0.f;
         if (rc == MP_OK && cudaEventElapsedTime(&ms, r->k0, r->k1) != cudaSuccess) rc = fail(MP_ERR_CUDA, "timing");
@@ -1595,7 +1639,7 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
         g->d = group_view(G->state + goff[i], rel[i].n);
         G->groups.push_back(g);
         Request* r = nullptr;
-        const int rc = prepare_request(ctx, g, &opts[i], s, &r, &hr[i], &md[i]);
+        const int rc = prepare_request(ctx, g, &opts[i], s, true, &r, &hr[i], &md[i]);
         if (rc != MP_OK) return bail(rc);
         r->graph_owned = true;
         cudaEventDestroy(r->k0);
@@ -1652,6 +1696,7 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
             e = cudaMemcpy(G->tables + o_req[p], rq.data(), sizeof(mp::Req) * rq.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess && !rq.empty())
             e = cudaMemcpy(G->tables + o_bst[p], bs.data(), sizeof(long long) * bs.size(), cudaMemcpyHostToDevice);
+        if (rq.size() == 1) bat[p].one = rq[0];
         bat[p].reqs = reinterpret_cast<const mp::Req*>(G->tables + o_req[p]);
         bat[p].starts = reinterpret_cast<const long long*>(G->tables + o_bst[p]);
         bat[p].n_reqs = (int)sel[p].size();
@@ -1665,10 +1710,11 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
     if ((e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking)) != cudaSuccess)
         return bail(cuda_fail(e, "mp_graph_create: stream"));
     e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
-    for (Request* r : G->reqs)
-        if (e == cudaSuccess) e = cudaMemsetAsync(r->d.counters, 0, sizeof(unsigned long long) * N_COUNTERS, cs);
-    for (int p = 0; p < 2 && e == cudaSuccess; ++p)
-        if (!sel[p].empty()) e = cudaMemsetAsync(bat[p].queue, 0, sizeof(unsigned long long), cs);
+    for (int p = 0; p < 2 && e == cudaSuccess; ++p) {
+        if (sel[p].empty()) continue;
+        e = mp::launch_zero_counters(bat[p], cs);
+        if (e == cudaSuccess) e = cudaMemsetAsync(bat[p].queue, 0, sizeof(unsigned long long), cs);
+    }
     if (e == cudaSuccess)
         e = mp::launch_release_boxes(fd, G->d_desc, reinterpret_cast<const long long*>(G->tables + o_st), n_reqs,
                                      starts[n_reqs], cs);

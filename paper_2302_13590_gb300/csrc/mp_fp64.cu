@@ -245,6 +245,7 @@ __global__ void k_release_explicit(DevField f, DevState st, long long n, const i
     if (q >= n) return;
     const long long c = cell[q];
     st.t[q] = t0 ? t0[q] : 0.0;
+    if (st.steps) st.steps[q] = 0u;
     if (c < 0 || c >= f.ncell) {
         st.cell[q] = -1; st.px[q] = 0.0; st.py[q] = 0.0; st.pz[q] = 0.0;
         st.status[q] = MP_ST_INVALID_RELEASE;
@@ -294,12 +295,22 @@ cudaError_t launch_release_explicit(const DevField& f, const DevState& st, long 
 // conversions and a branch in every helper: 1e6 particles, 200x200x20 cells,
 // 50 output times 27.2 -> 23.5 ms; 3e4 particles, endpoints 1.19 -> 1.05 ms;
 // 1000 particles, 50x50 cells 154 -> 135 us; the same bits.
+template <bool ONE_REQ>
 struct F64Engine {
+    static constexpr bool ONE = ONE_REQ;
     // blocks of 256 threads to keep resident per SM (0: no target; the
     // kernels are FP64-pipe bound)
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevField f;
     Batch b;
+
+    // descriptor of request r of the launch (ONE: the launch has one, by value)
+    __device__ __forceinline__ const Req& req(int r) const
+    {
+        if constexpr (ONE) return b.one;
+        else return b.reqs[r];
+    }
+
 
     struct State {
         int r;            // request of the particle within the launch
@@ -333,7 +344,7 @@ struct F64Engine {
     __device__ __forceinline__ void record(long long q, int kk, const State& s, double x, double y, double z,
                                            int st) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -356,7 +367,7 @@ struct F64Engine {
     // next time at which the step loop must leave its fast path
     __device__ __forceinline__ long long next_event(const State& s) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -372,7 +383,7 @@ struct F64Engine {
     __device__ __forceinline__ void load(int r, long long q, State& s) const
     {
         s.r = r;
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -436,12 +447,12 @@ struct F64Engine {
 
     __device__ __forceinline__ void rec_put(RecQ& Q, int slot, const State& s, long long q, int kk, int st) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
         (void)in; (void)o; (void)p;
-        Q.r[slot] = s.r;
+        if (!ONE) Q.r[slot] = s.r;
         Q.p0[slot] = s.x0; Q.p1[slot] = s.x1; Q.p2[slot] = s.x2;
         Q.t[slot] = s.t;   // tau = times[kk] - t is formed in rec_eval, where all 32 lanes take it
         Q.q[slot] = q;
@@ -453,7 +464,7 @@ struct F64Engine {
     // every axis (the same operations as an endpoint stop at that time)
     __device__ __forceinline__ void rec_eval(const RecQ& Q, int slot) const
     {
-        const Req& R = b.reqs[Q.r[slot]];
+        const Req& R = req(ONE ? 0 : Q.r[slot]);
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
         const int c = Q.c[slot], i = Q.i[slot], j = Q.j[slot], k = Q.k[slot];
@@ -482,7 +493,7 @@ struct F64Engine {
     template <bool TS>
     __device__ __forceinline__ void step(long long q, State& s, bool live, RecQ& Q, int& qcount) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -680,7 +691,7 @@ struct F64Engine {
     template <bool TS>
     __device__ __forceinline__ void finish(long long q, const State& s, unsigned long long* s_cnt) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -709,9 +720,22 @@ struct F64Engine {
         }
         // steps taken in this launch; a particle paused at the end of a flow
         // period is counted by the period it ends in
-        count_ended(b, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
+        count_ended(*this, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
     }
 };
+
+__global__ void k_zero_counters(const Req* reqs, int n)
+{
+    const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    if (i < n * N_COUNTERS) reqs[i / N_COUNTERS].o.counters[i % N_COUNTERS] = 0ULL;
+}
+
+cudaError_t launch_zero_counters(const Batch& b, cudaStream_t s)
+{
+    const long long words = (long long)b.n_reqs * N_COUNTERS;   // (below 2^31: fewer than 2^24 requests)
+    k_zero_counters<<<(unsigned)((words + 255) / 256), 256, 0, s>>>(b.reqs, b.n_reqs);
+    return cudaGetLastError();
+}
 
 // The tracking kernels keep a launch's device-time window in its first
 // request's counters; a batch's other requests get a copy.
@@ -735,8 +759,8 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s)
 cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                               int blocks_per_sm_cap, cudaStream_t s)
 {
-    F64Engine e{f, b};
-    return launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_reqs == 1) return launch_tracking(F64Engine<true>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    return launch_tracking(F64Engine<false>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
 }
 
 }  // namespace mp

@@ -197,9 +197,12 @@ struct Req {
 
 // A launch tracks the particles of one or more requests as one index space:
 // global particle g belongs to request r with starts[r] <= g < starts[r+1].
+// A launch of one request carries its descriptor by value (kernel parameters
+// sit in the constant bank: no table to copy, no load in front of each use).
 struct Batch {
-    const Req* reqs;             // [n_reqs], device
-    const long long* starts;     // [n_reqs + 1], device
+    Req one;                     // n_reqs == 1
+    const Req* reqs;             // n_reqs > 1: [n_reqs], device
+    const long long* starts;     // n_reqs > 1: [n_reqs + 1], device
     int n_reqs;
     long long n_total;
     int steps_per_fetch;
@@ -283,6 +286,8 @@ cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes,
                               int blocks_per_sm_cap, cudaStream_t s);
 cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                                int blocks_per_sm_cap, cudaStream_t s);
+// zero the counters of a batch's requests (n_reqs > 1)
+cudaError_t launch_zero_counters(const Batch& b, cudaStream_t s);
 // copy the first request's launch window into the other requests of a batch
 cudaError_t launch_spread_window(const Batch& b, cudaStream_t s);
 cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,

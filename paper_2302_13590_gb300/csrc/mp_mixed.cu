@@ -8,8 +8,9 @@ namespace mp {
 cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                                int blocks_per_sm_cap, cudaStream_t s)
 {
-    MixEngine<false> e{f, b};
-    return launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_reqs == 1)
+        return launch_tracking(MixEngine<false, true>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    return launch_tracking(MixEngine<false, false>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
 }
 
 }  // namespace mp

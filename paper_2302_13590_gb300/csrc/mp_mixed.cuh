@@ -41,8 +41,9 @@
 
 namespace mp {
 
-template <bool F64T>
+template <bool F64T, bool ONE_REQ>
 struct MixEngine {
+    static constexpr bool ONE = ONE_REQ;
     // blocks of 256 threads to keep resident per SM: the kernels are issue
     // bound, and without a target the compiler gives the static endpoint
     // kernel fewer registers than it needs (spills); four blocks (at most 64
@@ -50,6 +51,14 @@ struct MixEngine {
     static constexpr int min_blocks(bool dynamic, bool, bool pl) { return (!dynamic && !pl) ? 4 : 0; }
     DevField f;
     Batch b;
+
+    // descriptor of request r of the launch (ONE: the launch has one, by value)
+    __device__ __forceinline__ const Req& req(int r) const
+    {
+        if constexpr (ONE) return b.one;
+        else return b.reqs[r];
+    }
+
 
     struct State {
         int r;            // request of the particle within the launch
@@ -179,7 +188,7 @@ struct MixEngine {
     __device__ __forceinline__ void record(long long q, int kk, const State& s, double x, double y, double z,
                                            int st) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -201,7 +210,7 @@ struct MixEngine {
     // next event as a pair: the next output time or the stop time
     __device__ __forceinline__ void next_event(State& s) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -225,7 +234,7 @@ struct MixEngine {
     __device__ __forceinline__ void load(int r, long long q, State& s) const
     {
         s.r = r;
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -293,12 +302,12 @@ struct MixEngine {
 
     __device__ __forceinline__ void rec_put(RecQ& Q, int slot, const State& s, long long q, int kk, int st) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
         (void)in; (void)o; (void)p;
-        Q.r[slot] = s.r;
+        if (!ONE) Q.r[slot] = s.r;
         Q.x0[slot] = s.x0; Q.x1[slot] = s.x1; Q.x2[slot] = s.x2;
         if constexpr (F64T) {
             Q.tau[slot] = (float)(__ldg(o.times + kk) - s.t);
@@ -313,7 +322,7 @@ struct MixEngine {
 
     __device__ __forceinline__ void rec_eval(const RecQ& Q, int slot) const
     {
-        const Req& R = b.reqs[Q.r[slot]];
+        const Req& R = req(ONE ? 0 : Q.r[slot]);
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
         State r;
@@ -332,7 +341,7 @@ struct MixEngine {
     template <bool TS>
     __device__ __forceinline__ void step(long long q, State& s, bool live, RecQ& Q, int& qcount) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -480,7 +489,7 @@ struct MixEngine {
     template <bool TS>
     __device__ __forceinline__ void finish(long long q, const State& s, unsigned long long* s_cnt) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -517,7 +526,7 @@ struct MixEngine {
         }
         // steps taken in this launch; a particle paused at the end of a flow
         // period is counted by the period it ends in
-        count_ended(b, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
+        count_ended(*this, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
     }
 };
 

@@ -9,8 +9,9 @@ namespace mp {
 cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                                     int blocks_per_sm_cap, cudaStream_t s)
 {
-    MixEngine<true> e{f, b};
-    return launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_reqs == 1)
+        return launch_tracking(MixEngine<true, true>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    return launch_tracking(MixEngine<true, false>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
 }
 
 }  // namespace mp

@@ -7,10 +7,9 @@
 // pool behind its back.  mp_track_noalloc serves them: the caller passes
 // every input and output buffer, and the only other device memory the call
 // uses is the small file-scope array below, which every GPU that loads this
-// library holds until the process exits.  The call does copy its small
-// host-side inputs (output times, the request descriptor) with
-// cudaMemcpyAsync from pageable host memory, which may block the calling
-// thread until the stream reaches the copy.
+// library holds until the process exits.  The call does copy its output
+// times with cudaMemcpyAsync from pageable host memory, which may block the
+// calling thread until the stream reaches the copy.
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -23,9 +22,8 @@ using namespace mp;
 namespace {
 
 // queue head, reduction counters, a copy of the output times and the same
-// times as FP32 pairs, and the launch's one-entry request table
-constexpr int kReqWords = (int)((sizeof(Req) + 2 * sizeof(long long) + 7) / 8);
-constexpr int kScratchWords = 8 + N_COUNTERS + 2 * MP_NOALLOC_MAX_TIMES + kReqWords;
+// times as FP32 pairs
+constexpr int kScratchWords = 8 + N_COUNTERS + 2 * MP_NOALLOC_MAX_TIMES;
 static __device__ __align__(256) unsigned long long g_noalloc_scratch[kScratchWords];
 
 constexpr int kMaxDevices = 64;
@@ -116,8 +114,6 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
         }
     }
     if (e != cudaSuccess) return na_fail(MP_ERR_CUDA, std::string("mp_track_noalloc: ") + cudaGetErrorString(e));
-    Req* dreq = reinterpret_cast<Req*>(scratch + 8 + N_COUNTERS + 2 * MP_NOALLOC_MAX_TIMES);
-    long long* dstarts = reinterpret_cast<long long*>(reinterpret_cast<char*>(dreq) + sizeof(Req));
     DevState st{a->cell, a->px, a->py, a->pz, a->t, a->status, nullptr, nullptr, nullptr};
     DevOut d{};
     d.cell = ep.cell; d.x = ep.x; d.y = ep.y; d.z = ep.z; d.px = ep.px; d.py = ep.py; d.pz = ep.pz; d.t = ep.t;
@@ -141,17 +137,10 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     split_ff(p.t_stop, p.tstop_hi, p.tstop_lo);
     const int block = o->block > 0 ? o->block : 128;
     const DevField& fd = *mp::field_device_view(f);
-    Req hreq;
-    hreq.in = st;
-    hreq.o = d;
-    hreq.p = p;
-    const long long hstarts[2] = {0, a->n};
-    e = cudaMemcpyAsync(dreq, &hreq, sizeof(Req), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dstarts, hstarts, sizeof(hstarts), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return na_fail(MP_ERR_CUDA, std::string("mp_track_noalloc: ") + cudaGetErrorString(e));
     Batch b{};
-    b.reqs = dreq;
-    b.starts = dstarts;
+    b.one.in = st;
+    b.one.o = d;
+    b.one.p = p;
     b.n_reqs = 1;
     b.n_total = a->n;
     b.steps_per_fetch = p.steps_per_fetch;

@@ -46,16 +46,17 @@ template <class E>
 __device__ __forceinline__ void flush_counters(const E& e, unsigned long long* s_cnt)
 {
     __syncthreads();
-    if (e.b.n_reqs != 1) return;
-    unsigned long long* dst = e.b.reqs[0].o.counters;
+    if (!E::ONE) return;
+    unsigned long long* dst = e.req(0).o.counters;
     for (int i = threadIdx.x; i < COUNTER_ERR; i += blockDim.x)
         if (s_cnt[i]) atomicAdd(dst + i, s_cnt[i]);
 }
 
-__device__ __forceinline__ void count_ended(const Batch& b, int r, unsigned steps, int st,
+template <class E>
+__device__ __forceinline__ void count_ended(const E& e, int r, unsigned steps, int st,
                                             unsigned long long* s_cnt, bool count_status)
 {
-    unsigned long long* c = b.n_reqs == 1 ? s_cnt : b.reqs[r].o.counters;
+    unsigned long long* c = E::ONE ? s_cnt : e.req(r).o.counters;
     atomicAdd(c + COUNTER_STEPS, (unsigned long long)steps);
     if (count_status) atomicAdd(c + COUNTER_STATUS + (st & 7), 1ULL);
 }
@@ -65,7 +66,7 @@ __device__ __forceinline__ void count_ended(const Batch& b, int r, unsigned step
 template <class E, class S>
 __device__ __forceinline__ bool paused(const E& e, const S& s)
 {
-    return (s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP) && !e.b.reqs[s.r].p.last;
+    return (s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP) && !e.req(s.r).p.last;
 }
 
 // The launch's device-time window (global timer, ns), kept in the first
@@ -77,25 +78,32 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-__device__ __forceinline__ void window_begin(const Batch& b)
+template <class E>
+__device__ __forceinline__ void window_begin(const E& e)
 {
-    if (threadIdx.x == 0) atomicMax(b.reqs[0].o.counters + COUNTER_T_BEGIN, ~global_ns());
+    if (threadIdx.x == 0) atomicMax(e.req(0).o.counters + COUNTER_T_BEGIN, ~global_ns());
 }
 
-__device__ __forceinline__ void window_end(const Batch& b)
+template <class E>
+__device__ __forceinline__ void window_end(const E& e)
 {
-    if (threadIdx.x == 0) atomicMax(b.reqs[0].o.counters + COUNTER_T_END, global_ns());
+    if (threadIdx.x == 0) atomicMax(e.req(0).o.counters + COUNTER_T_END, global_ns());
 }
 
-// request of global particle index g (starts ascending, starts[0] = 0)
-__device__ __forceinline__ int request_of(const Batch& b, long long g)
+// request of global particle index g (starts ascending, starts[0] = 0) and
+// the particle's index in it
+template <class E>
+__device__ __forceinline__ int request_of(const E& e, long long g, long long& q)
 {
-    int lo = 0, hi = b.n_reqs - 1;
+    q = g;
+    if (E::ONE) return 0;
+    int lo = 0, hi = e.b.n_reqs - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (__ldg(b.starts + mid) <= g) lo = mid;
+        if (__ldg(e.b.starts + mid) <= g) lo = mid;
         else hi = mid - 1;
     }
+    q = g - __ldg(e.b.starts + lo);
     return lo;
 }
 
@@ -175,9 +183,9 @@ __device__ __forceinline__ void tail_fill(const E& e, const typename E::State& s
         mask &= mask - 1;
         const double bx = __shfl_sync(FULL, x, L), by = __shfl_sync(FULL, y, L), bz = __shfl_sync(FULL, z, L);
         const int c = __shfl_sync(FULL, s.c, L), st = __shfl_sync(FULL, s.st, L), kn = __shfl_sync(FULL, s.kn, L);
-        const int r = __shfl_sync(FULL, s.r, L);
+        const int r = E::ONE ? 0 : __shfl_sync(FULL, s.r, L);
         const long long qq = __shfl_sync(FULL, q, L);
-        const Req& R = e.b.reqs[r];
+        const Req& R = e.req(r);
         const int nt = R.p.n_times;
         mp_ts_record* ts = R.o.ts;
         const long long n = R.p.n;
@@ -224,15 +232,15 @@ __device__ __forceinline__ void pl_flush(const E& e, PathQ& Q, int& pcount)
     for (int base = 0; base < pcount; base += 32) {
         const int i = base + lane;
         const bool has = i < pcount;
-        const int r = has ? Q.r[i] : -1;
-        const unsigned peers = __match_any_sync(FULL, r);
-        const int leader = __ffs(peers) - 1;
+        const int r = has ? (E::ONE ? 0 : Q.r[i]) : -1;
+        const unsigned peers = E::ONE ? __ballot_sync(FULL, has) : __match_any_sync(FULL, r);
+        const int leader = (__ffs(peers) - 1) & 31;
         unsigned long long pos = 0;
         if (has && lane == leader)
-            pos = atomicAdd(e.b.reqs[r].o.counters + COUNTER_PATH, (unsigned long long)__popc(peers));
+            pos = atomicAdd(e.req(r).o.counters + COUNTER_PATH, (unsigned long long)__popc(peers));
         pos = __shfl_sync(FULL, pos, leader) + (unsigned long long)__popc(peers & lt);
         if (has) {
-            const DevOut& o = e.b.reqs[r].o;
+            const DevOut& o = e.req(r).o;
             if ((long long)pos < o.path_cap) store_path(o.path + pos, Q, i);
         }
     }
@@ -255,7 +263,8 @@ __device__ __forceinline__ void pl_push(const E& e, PathQ& Q, int& pcount, const
         double x, y, z, t;
         e.path_point(s, x, y, z, t);
         Q.x[slot] = x; Q.y[slot] = y; Q.z[slot] = z; Q.t[slot] = t;
-        Q.q[slot] = (int)q; Q.c[slot] = s.c; Q.r[slot] = s.r;
+        Q.q[slot] = (int)q; Q.c[slot] = s.c;
+        if (!E::ONE) Q.r[slot] = s.r;
         Q.seq[slot] = s.steps;
         Q.st[slot] = (unsigned char)st;
     }
@@ -269,7 +278,7 @@ __device__ __forceinline__ void pl_push(const E& e, PathQ& Q, int& pcount, const
 template <class E, class S>
 __device__ __forceinline__ bool path_start(const E& e, const S& s)
 {
-    const TrackParams& p = e.b.reqs[s.r].p;
+    const TrackParams& p = e.req(s.r).p;
     return p.pathline && !p.cont && s.st != ST_SKIP && s.c >= 0;
 }
 
@@ -279,7 +288,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_sta
     __shared__ unsigned long long s_cnt[N_COUNTERS];
     typename E::RecQ* s_q = reinterpret_cast<typename E::RecQ*>(s_dyn);
     for (int i = threadIdx.x; i < N_COUNTERS; i += blockDim.x) s_cnt[i] = 0ULL;
-    window_begin(e.b);
+    window_begin(e);
     __syncthreads();
     const unsigned FULL = 0xffffffffu;
     typename E::RecQ& Q = s_q[TS ? (threadIdx.x >> 5) : 0];
@@ -295,8 +304,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_sta
     s.c = -1;
     bool live = false, ended = false, loaded = false;
     if (g < e.b.n_total) {
-        const int r = request_of(e.b, g);
-        q = g - __ldg(e.b.starts + r);
+        const int r = request_of(e, g, q);
         e.template load<TS>(r, q, s);
         live = s.st == MP_ST_ACTIVE;
         ended = !live && s.st != ST_SKIP;
@@ -308,7 +316,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_sta
     while (__any_sync(FULL, live)) {
         const unsigned before = s.steps;
         e.template step<TS>(q, s, live, Q, qcount);
-        if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.b.reqs[s.r].p.pathline, s.st);
+        if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.req(s.r).p.pathline, s.st);
         ended = live && s.st != MP_ST_ACTIVE;
         if (TS) tail_fill(e, s, q, ended && !paused(e, s));
         if (ended) {
@@ -319,7 +327,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_sta
     if (TS) rq_drain(e, Q, qcount, true);
     if (PL) pl_flush(e, P, pcount);
     flush_counters(e, s_cnt);
-    window_end(e.b);
+    window_end(e);
 }
 
 template <class E, bool TS, bool PL>
@@ -328,7 +336,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     __shared__ unsigned long long s_cnt[N_COUNTERS];
     typename E::RecQ* s_q = reinterpret_cast<typename E::RecQ*>(s_dyn);
     for (int i = threadIdx.x; i < N_COUNTERS; i += blockDim.x) s_cnt[i] = 0ULL;
-    window_begin(e.b);
+    window_begin(e);
     __syncthreads();
     typename E::RecQ& Q = s_q[TS ? (threadIdx.x >> 5) : 0];
     PathQ* s_p = reinterpret_cast<PathQ*>(s_dyn + (TS ? sizeof(typename E::RecQ) * (blockDim.x >> 5) : 0));
@@ -359,8 +367,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
             if (!live) {
                 const unsigned long long qq = base + __popc(idle & lt_mask);
                 if (qq < n) {
-                    const int r = request_of(e.b, (long long)qq);
-                    q = (long long)qq - __ldg(e.b.starts + r);
+                    const int r = request_of(e, (long long)qq, q);
                     e.template load<TS>(r, q, s);
                     live = s.st == MP_ST_ACTIVE;
                     ended = !live && s.st != ST_SKIP;
@@ -378,7 +385,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
         for (int it = 0; it < S; ++it) {
             const unsigned before = s.steps;
             e.template step<TS>(q, s, live, Q, qcount);
-            if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.b.reqs[s.r].p.pathline, s.st);
+            if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.req(s.r).p.pathline, s.st);
             ended = live && s.st != MP_ST_ACTIVE;
             if (TS) tail_fill(e, s, q, ended && !paused(e, s));
             if (ended) {
@@ -390,7 +397,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     if (TS) rq_drain(e, Q, qcount, true);
     if (PL) pl_flush(e, P, pcount);
     flush_counters(e, s_cnt);
-    window_end(e.b);
+    window_end(e);
 }
 
 // One variant of the tracking kernel: opt in to more than 48 KB of dynamic

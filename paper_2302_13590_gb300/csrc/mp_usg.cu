@@ -115,6 +115,7 @@ __global__ void k_release_explicit_usg(DevUsg u, DevState st, long long n, const
     if (q >= n) return;
     const long long c = cell[q];
     st.t[q] = t0 ? t0[q] : 0.0;
+    if (st.steps) st.steps[q] = 0u;
     if (c < 0 || c >= u.ncell) {
         st.cell[q] = -1; st.px[q] = 0.0; st.py[q] = 0.0; st.pz[q] = 0.0;
         st.status[q] = MP_ST_INVALID_RELEASE;
@@ -142,10 +143,20 @@ cudaError_t launch_release_explicit_usg(const DevUsg& u, const DevState& st, lon
 // tracking engine
 // ---------------------------------------------------------------------------
 
+template <bool ONE_REQ>
 struct UsgEngine {
+    static constexpr bool ONE = ONE_REQ;
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevUsg u;
     Batch b;
+
+    // descriptor of request r of the launch (ONE: the launch has one, by value)
+    __device__ __forceinline__ const Req& req(int r) const
+    {
+        if constexpr (ONE) return b.one;
+        else return b.reqs[r];
+    }
+
 
     template <class T>
     __device__ __forceinline__ static T sel3(int a, T x, T y, T z)
@@ -175,7 +186,7 @@ struct UsgEngine {
     __device__ __forceinline__ void record(long long q, int kk, const State& s, double x, double y, double z,
                                            int st) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         store_record(R.o.ts + (long long)kk * R.p.n + q, x, y, z, s.c, st);
     }
 
@@ -189,7 +200,7 @@ struct UsgEngine {
 
     __device__ __forceinline__ long long next_event(const State& s) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const double tk = s.kn < R.p.n_times ? __ldg(R.o.times + s.kn) : CUDART_INF;
         return bound_key(ge_d(tk, R.p.t_stop) ? R.p.t_stop : tk);
     }
@@ -198,7 +209,7 @@ struct UsgEngine {
     __device__ __forceinline__ void load(int r, long long q, State& s) const
     {
         s.r = r;
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -251,8 +262,8 @@ struct UsgEngine {
 
     __device__ __forceinline__ void rec_put(RecQ& Q, int slot, const State& s, long long q, int kk, int st) const
     {
-        const Req& R = b.reqs[s.r];
-        Q.r[slot] = s.r;
+        const Req& R = req(s.r);
+        if (!ONE) Q.r[slot] = s.r;
         Q.p0[slot] = s.x0; Q.p1[slot] = s.x1; Q.p2[slot] = s.x2;
         Q.tau[slot] = __ldg(R.o.times + kk) - s.t;
         Q.q[slot] = q;
@@ -262,7 +273,7 @@ struct UsgEngine {
 
     __device__ __forceinline__ void rec_eval(const RecQ& Q, int slot) const
     {
-        const Req& R = b.reqs[Q.r[slot]];
+        const Req& R = req(ONE ? 0 : Q.r[slot]);
         const int c = Q.c[slot];
         const UsgCell& k = u.cell[c];
         const UsgGeo& g = u.geo[c];
@@ -365,7 +376,7 @@ struct UsgEngine {
     template <bool TS>
     __device__ __forceinline__ void step(long long q, State& s, bool live, RecQ& Q, int& qcount) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
         enum { P_NONE, P_CROSS, P_TIME, P_NOEXIT, P_CAPTURE };
@@ -579,7 +590,7 @@ struct UsgEngine {
     template <bool TS>
     __device__ __forceinline__ void finish(long long q, const State& s, unsigned long long* s_cnt) const
     {
-        const Req& R = b.reqs[s.r];
+        const Req& R = req(s.r);
         const DevState& in = R.in;
         const DevOut& o = R.o;
         const TrackParams& p = R.p;
@@ -605,15 +616,15 @@ struct UsgEngine {
                 in.exit_face[q] = (uint8_t)s.ef;
             }
         }
-        count_ended(b, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
+        count_ended(*this, s.r, s.steps - base, s.st, s_cnt, p.last || !(s.st == MP_ST_TIME || s.st == MP_ST_STEP_CAP));
     }
 };
 
 cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block,
                              int blocks_per_sm_cap, cudaStream_t s)
 {
-    UsgEngine e{u, b};
-    return launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_reqs == 1) return launch_tracking(UsgEngine<true>{u, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    return launch_tracking(UsgEngine<false>{u, b}, modes, schedule, block, blocks_per_sm_cap, s);
 }
 
 }  // namespace mp
