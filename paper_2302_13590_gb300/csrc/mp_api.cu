@@ -1207,6 +1207,19 @@ int copy_out(void* dst, const void* src, size_t bytes, bool dev, cudaStream_t s)
     return MP_OK;
 }
 
+// memory that a kernel on `device` can write: its own or managed memory
+// (anything else goes through cudaMemcpyAsync, as pinned host memory or
+// another device's)
+bool kernel_can_write(const void* p, int device)
+{
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (a.type == cudaMemoryTypeDevice && a.device == device) || a.type == cudaMemoryTypeManaged;
+}
+
 int prepare_read(mp_ctx* ctx, Request* r, uint32_t flags, cudaStream_t s)
 {
     if (flags & MP_DEVICE_PTR) {
@@ -1236,18 +1249,23 @@ int mp_get_endpoints(mp_ctx* ctx, mp_req id, const mp_endpoints* out, uint32_t f
     if (rc != MP_OK) return rc;
     const bool dev = (flags & MP_DEVICE_PTR) != 0;
     const size_t n = (size_t)r->n;
-    if ((rc = copy_out(out->cell, r->d.cell, 4 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->x, r->d.x, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->y, r->d.y, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->z, r->d.z, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->px, r->d.px, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->py, r->d.py, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->pz, r->d.pz, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->t, r->d.t, 8 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->status, r->d.status, n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->steps, r->d.steps, 4 * n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->exit_face, r->d.exit_face, n, dev, s)) != MP_OK) return rc;
-    if ((rc = copy_out(out->hash, r->d.hash, 8 * n, dev, s)) != MP_OK) return rc;
+    const struct { void* dst; const void* src; size_t bytes; } arrays[] = {
+        {out->cell, r->d.cell, 4 * n},     {out->x, r->d.x, 8 * n},   {out->y, r->d.y, 8 * n},
+        {out->z, r->d.z, 8 * n},           {out->px, r->d.px, 8 * n}, {out->py, r->d.py, 8 * n},
+        {out->pz, r->d.pz, 8 * n},         {out->t, r->d.t, 8 * n},   {out->status, r->d.status, n},
+        {out->steps, r->d.steps, 4 * n},   {out->exit_face, r->d.exit_face, n},
+        {out->hash, r->d.hash, 8 * n}};
+    mp::CopyList list{};
+    for (const auto& x : arrays) {
+        if (!x.dst || x.bytes == 0) continue;
+        if (dev && kernel_can_write(x.dst, ctx->device)) {
+            list.a[list.n++] = mp::CopyItem{x.dst, x.src, x.bytes};
+            list.most = std::max<unsigned long long>(list.most, x.bytes);
+        } else if ((rc = copy_out(x.dst, x.src, x.bytes, dev, s)) != MP_OK) {
+            return rc;
+        }
+    }
+    MP_CUDA(mp::launch_copy_list(list, s), "mp_get_endpoints: copy");
     return MP_OK;
 }
 

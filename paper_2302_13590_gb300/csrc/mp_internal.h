@@ -293,6 +293,19 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s);
 cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                                int blocks_per_sm_cap, cudaStream_t s);
 
+// device-to-device copies of a request's arrays into the caller's, as one launch
+struct CopyItem {
+    void* dst;
+    const void* src;
+    unsigned long long bytes;
+};
+struct CopyList {
+    CopyItem a[12];
+    int n;
+    unsigned long long most;   // the largest item's bytes
+};
+cudaError_t launch_copy_list(const CopyList& c, cudaStream_t s);
+
 // Host helpers shared by the entry points: the calling thread's error
 // message (what mp_last_error returns) and a loaded field's device view.
 void set_last_error(const char* msg);
