@@ -152,6 +152,8 @@ struct mp_ctx {
     std::mutex mu;
     std::mutex host_mu;                             // one mp_track_host at a time per context
     cudaStream_t host_st[2] = {nullptr, nullptr};   // its two streams, made on first use
+    cudaStream_t load_st = nullptr;                 // field loads and frees
+    cudaMemPool_t field_pool = nullptr;             // fields and their load's scratch
     std::map<TuneKey, mp_tuning> tuned;
     std::map<int64_t, Request*> reqs;
     std::set<mp_field*> fields;
@@ -196,37 +198,45 @@ int read_counters(Request* r, unsigned long long* h)
     return MP_OK;
 }
 
-// The balance report from per-cell (inflow, outflow) and ibound, in cell order.
-mp_balance reduce_balance(const std::vector<double2>& io, const int8_t* ib, long long ncell)
+// Device memory of fields comes from a pool of the context that keeps at most
+// this much when fields are freed: the next load of a transient model's field
+// then reuses mapped memory (cudaMalloc and cudaFree of a 200x200x20 field's
+// 136 MB took 1.1 ms).  What is above goes back at the next synchronisation,
+// the rest with the context.
+constexpr uint64_t FIELD_POOL_KEEP = 1ULL << 30;
+
+// the report of a reduced balance; the sink cells' extractions are read and
+// summed in cell order
+cudaError_t balance_report(mp_ctx* ctx, const BalancePart& t, const double2* inout, long long ncell,
+                           const BalancePart* parts, mp_balance* out)
 {
     mp_balance b{};
     b.max_abs_cell = -1;
-    for (long long c = 0; c < ncell; ++c) {
-        const double in = io[(size_t)c].x, out = io[(size_t)c].y;
-        if (ib[c] == 1) {
-            const double r = std::fabs(in - out);
-            if (b.max_abs_cell < 0 || r > b.max_abs_residual) {
-                b.max_abs_residual = r;
-                b.max_abs_cell = c;
-            }
-            if (in > 0.0) b.max_rel_residual = std::max(b.max_rel_residual, r / in);
-            b.active_cells++;
-        } else if (ib[c] == 2) {
-            b.sink_extraction += in - out;
-            b.sink_cells++;
-        }
+    b.active_cells = t.active;
+    b.sink_cells = t.sinks;
+    if (t.first >= 0) {
+        // (a first residual that is not a number stays the maximum)
+        const bool nan = std::isnan(t.r_first);
+        b.max_abs_residual = nan ? t.r_first : t.max_abs;
+        b.max_abs_cell = nan ? t.first : t.cell;
+        b.max_rel_residual = t.max_rel;
     }
-    return b;
-}
-
-// per-cell (inflow, outflow) from the device, reduced on the host
-int balance_from_device(const double2* dio, const int8_t* host_ib, long long ncell, mp_balance* out)
-{
-    std::vector<double2> io((size_t)ncell);
-    if (ncell > 0)
-        MP_CUDA(cudaMemcpy(io.data(), dio, sizeof(double2) * (size_t)ncell, cudaMemcpyDeviceToHost), "balance copy");
-    *out = reduce_balance(io, host_ib, ncell);
-    return MP_OK;
+    if (t.sinks > 0) {
+        const cudaStream_t s = ctx->load_st;
+        std::vector<double> x((size_t)t.sinks);
+        double* packed = nullptr;
+        cudaError_t e = cudaMallocFromPoolAsync(&packed, sizeof(double) * x.size(), ctx->field_pool, s);
+        if (e != cudaSuccess) return e;
+        e = launch_balance_sinks(inout, ncell, parts, packed, s);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(x.data(), packed, sizeof(double) * x.size(), cudaMemcpyDeviceToHost, s);
+        cudaFreeAsync(packed, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return e;
+        for (double v : x) b.sink_extraction += v;
+    }
+    *out = b;
+    return cudaSuccess;
 }
 
 }  // namespace
@@ -257,6 +267,22 @@ int mp_ctx_create(int device, mp_ctx** out)
     }
     mp_ctx* c = new mp_ctx();
     c->device = device;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaError_t e = cudaStreamCreateWithFlags(&c->load_st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemPoolCreate(&c->field_pool, &props);
+    if (e == cudaSuccess) {
+        uint64_t keep = FIELD_POOL_KEEP;
+        e = cudaMemPoolSetAttribute(c->field_pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
+    if (e != cudaSuccess) {
+        if (c->field_pool) cudaMemPoolDestroy(c->field_pool);
+        if (c->load_st) cudaStreamDestroy(c->load_st);
+        delete c;
+        return cuda_fail(e, "mp_ctx_create: field pool");
+    }
     *out = c;
     return MP_OK;
 }
@@ -280,6 +306,8 @@ int mp_ctx_destroy(mp_ctx* ctx)
     cudaDeviceSynchronize();
     for (cudaStream_t x : ctx->host_st)
         if (x) cudaStreamDestroy(x);
+    cudaStreamDestroy(ctx->load_st);
+    cudaMemPoolDestroy(ctx->field_pool);
     delete ctx;
     return MP_OK;
 }
@@ -304,7 +332,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     MP_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
 
     const long long nqx = nl * nr * (nc + 1), nqy = nl * (nr + 1) * nc, nqz = (nl + 1) * nr * nc;
-    // persistent layout
+    // persistent layout; the axes' arrays are one block, made on the host
     size_t off = 0;
     const size_t o_r64 = off; off = align256(off + sizeof(CellF64) * ncell);
     const size_t o_r32 = off; off = align256(off + sizeof(CellF32) * ncell);
@@ -317,59 +345,61 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     const size_t o_zf = off; off = align256(off + sizeof(double) * (nl + 1));
     const size_t o_ib = off; off = align256(off + ncell);
     const size_t o_sf = off; off = align256(off + sizeof(double) * ncell);
-    const size_t o_flag = off; off = align256(off + sizeof(unsigned));
     const size_t persistent = off;
     const bool dev_in = (d->flags & MP_DEVICE_PTR) != 0;
-    // staging for host inputs (freed once the records are built)
+    // scratch (freed once the records are built): what comes back to the
+    // host, the balance, and staging for host inputs
+    struct Back { BalancePart total; unsigned flags; };
     size_t soff = 0;
+    const size_t o_back = soff; soff = align256(soff + sizeof(Back));
+    const size_t o_part = soff; soff = align256(soff + sizeof(BalancePart) * BALANCE_BLOCKS);
+    const size_t o_io = soff; soff = align256(soff + sizeof(double2) * ncell);
     const size_t o_qx = soff; soff = align256(soff + (dev_in ? 0 : sizeof(double) * nqx));
     const size_t o_qy = soff; soff = align256(soff + (dev_in ? 0 : sizeof(double) * nqy));
     const size_t o_qz = soff; soff = align256(soff + (dev_in ? 0 : sizeof(double) * nqz));
     const size_t o_por = soff; soff = align256(soff + (dev_in ? 0 : sizeof(double) * ncell));
 
+    const cudaStream_t s = ctx->load_st;
     char* buf = nullptr;
     char* stage = nullptr;
-    if (cudaMalloc(&buf, persistent) != cudaSuccess || (!dev_in && cudaMalloc(&stage, soff) != cudaSuccess)) {
+    if (cudaMallocFromPoolAsync(&buf, persistent, ctx->field_pool, s) != cudaSuccess ||
+        cudaMallocFromPoolAsync(&stage, soff, ctx->field_pool, s) != cudaSuccess) {
         cudaGetLastError();
-        if (buf) cudaFree(buf);
+        if (buf) cudaFreeAsync(buf, s);
         return fail(MP_ERR_OOM, "mp_field_load: device allocation failed");
     }
-    auto cleanup = [&](int rc) { cudaFree(buf); if (stage) cudaFree(stage); return rc; };
-    std::vector<double> xf(nc + 1), yf(nr + 1), zf(nl + 1);
-    xf[0] = d->origin[0];
-    for (long long a = 0; a < nc; ++a) xf[a + 1] = xf[a] + d->delr[a];
-    yf[0] = d->origin[1];
-    for (long long a = 0; a < nr; ++a) yf[a + 1] = yf[a] + d->delc[a];
-    zf[0] = d->origin[2];
-    for (long long a = 0; a < nl; ++a) zf[a + 1] = zf[a] + d->dz[a];
-
-    std::vector<AxisCell> axc;
-    axc.reserve((size_t)(nc + nr + nl));
+    auto fin = [&](int rc) {
+        cudaFreeAsync(stage, s);
+        cudaFreeAsync(buf, s);
+        cudaStreamSynchronize(s);
+        return rc;
+    };
+    std::vector<char> axes(o_ib - o_delr, 0);
+    auto host = [&](size_t o) { return reinterpret_cast<double*>(axes.data() + (o - o_delr)); };
+    memcpy(host(o_delr), d->delr, sizeof(double) * nc);
+    memcpy(host(o_delc), d->delc, sizeof(double) * nr);
+    memcpy(host(o_dz), d->dz, sizeof(double) * nl);
+    AxisCell* axc = reinterpret_cast<AxisCell*>(host(o_ax));
     int no_screen = 0;
-    auto add_axis = [&](const double* D, long long m) {
+    auto add_axis = [&](const double* D, long long m, double org, double* face) {
+        face[0] = org;
         for (long long a = 0; a < m; ++a) {
-            axc.push_back(AxisCell{D[a], host_f32_trunc(D[a]), 0.0f});
+            face[a + 1] = face[a] + D[a];
+            *axc++ = AxisCell{D[a], host_f32_trunc(D[a]), 0.0f};
             if (D[a] > SCREEN_MAX_D) no_screen = 1;
         }
     };
-    add_axis(d->delr, nc);
-    add_axis(d->delc, nr);
-    add_axis(d->dz, nl);
+    add_axis(d->delr, nc, d->origin[0], host(o_xf));
+    add_axis(d->delc, nr, d->origin[1], host(o_yf));
+    add_axis(d->dz, nl, d->origin[2], host(o_zf));
 
-    cudaStream_t s = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return cleanup(cuda_fail(e, "cudaStreamCreate"));
-    auto fin = [&](int rc) {
-        cudaStreamSynchronize(s);
-        cudaStreamDestroy(s);
-        return cleanup(rc);
-    };
     const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
     const cudaMemcpyKind in_kind = dev_in ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     const double* qx = dev_in ? d->qx : reinterpret_cast<double*>(stage + o_qx);
     const double* qy = dev_in ? d->qy : reinterpret_cast<double*>(stage + o_qy);
     const double* qz = dev_in ? d->qz : reinterpret_cast<double*>(stage + o_qz);
     const double* por = dev_in ? d->porosity : reinterpret_cast<double*>(stage + o_por);
+    cudaError_t e = cudaSuccess;
     if (!dev_in) {
         if ((e = cudaMemcpyAsync(stage + o_qx, d->qx, sizeof(double) * nqx, h2d, s)) != cudaSuccess ||
             (e = cudaMemcpyAsync(stage + o_qy, d->qy, sizeof(double) * nqy, h2d, s)) != cudaSuccess ||
@@ -377,71 +407,52 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
             (e = cudaMemcpyAsync(stage + o_por, d->porosity, sizeof(double) * ncell, h2d, s)) != cudaSuccess)
             return fin(cuda_fail(e, "mp_field_load: upload"));
     }
+    Back* back = reinterpret_cast<Back*>(stage + o_back);
     if ((e = cudaMemcpyAsync(buf + o_ib, d->ibound, ncell, in_kind, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_delr, d->delr, sizeof(double) * nc, h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_delc, d->delc, sizeof(double) * nr, h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_dz, d->dz, sizeof(double) * nl, h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_ax, axc.data(), sizeof(AxisCell) * axc.size(), h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_xf, xf.data(), sizeof(double) * (nc + 1), h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_yf, yf.data(), sizeof(double) * (nr + 1), h2d, s)) != cudaSuccess ||
-        (e = cudaMemcpyAsync(buf + o_zf, zf.data(), sizeof(double) * (nl + 1), h2d, s)) != cudaSuccess ||
-        (e = cudaMemsetAsync(buf + o_flag, 0, sizeof(unsigned), s)) != cudaSuccess)
+        (e = cudaMemcpyAsync(buf + o_delr, axes.data(), axes.size(), h2d, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(back, 0, sizeof(Back), s)) != cudaSuccess)
         return fin(cuda_fail(e, "mp_field_load: upload"));
-    unsigned* dflag = reinterpret_cast<unsigned*>(buf + o_flag);
-    if ((e = launch_validate(qx, nqx, qy, nqy, qz, nqz, por, reinterpret_cast<int8_t*>(buf + o_ib), ncell, dflag,
-                             s)) != cudaSuccess)
-        return fin(cuda_fail(e, "mp_field_load: validate"));
-    unsigned hflag = 0;
-    if ((e = cudaMemcpyAsync(&hflag, dflag, sizeof(unsigned), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
+    DevField v{};
+    v.nlay = (int)nl; v.nrow = (int)nr; v.ncol = (int)nc;
+    v.ncell = ncell;
+    v.rec64 = reinterpret_cast<CellF64*>(buf + o_r64);
+    v.rec32 = reinterpret_cast<CellF32*>(buf + o_r32);
+    v.delr = reinterpret_cast<double*>(buf + o_delr);
+    v.delc = reinterpret_cast<double*>(buf + o_delc);
+    v.dz = reinterpret_cast<double*>(buf + o_dz);
+    v.ax = reinterpret_cast<AxisCell*>(buf + o_ax);
+    v.no_screen = no_screen;
+    v.xf = reinterpret_cast<double*>(buf + o_xf);
+    v.yf = reinterpret_cast<double*>(buf + o_yf);
+    v.zf = reinterpret_cast<double*>(buf + o_zf);
+    v.ibound = reinterpret_cast<int8_t*>(buf + o_ib);
+    v.sinkfrac = reinterpret_cast<double*>(buf + o_sf);
+    v.m_ncol = div_magic((unsigned)nc);
+    v.m_nrow = div_magic((unsigned)nr);
+    // validation, records and balance in one go (the records of a field that
+    // turns out invalid are built, in bounds, and dropped), then one wait
+    double2* dio = reinterpret_cast<double2*>(stage + o_io);
+    BalancePart* parts = reinterpret_cast<BalancePart*>(stage + o_part);
+    Back got{};
+    if ((e = launch_validate(qx, nqx, qy, nqy, qz, nqz, por, v.ibound, ncell, &back->flags, s)) != cudaSuccess ||
+        (e = launch_build_records(v, reinterpret_cast<CellF64*>(buf + o_r64), reinterpret_cast<CellF32*>(buf + o_r32),
+                                  reinterpret_cast<double*>(buf + o_sf), dio, qx, qy, qz, por, s)) != cudaSuccess ||
+        (e = launch_balance(dio, v.ibound, ncell, parts, &back->total, s)) != cudaSuccess ||
+        (e = cudaMemcpyAsync(&got, back, sizeof(Back), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
-        return fin(cuda_fail(e, "mp_field_load: validate"));
-    if (hflag & 1u) return fin(fail(MP_ERR_NONFINITE, "mp_field_load: non-finite face flow"));
-    if (hflag & 2u) return fin(fail(MP_ERR_NONFINITE, "mp_field_load: porosity outside (0, 1] in an active cell"));
-    if (hflag & 4u) return fin(fail(MP_ERR_INVALID_ARG, "mp_field_load: ibound outside {-1, 0, 1, 2}"));
+        return fin(cuda_fail(e, "mp_field_load: build records"));
+    if (got.flags & 1u) return fin(fail(MP_ERR_NONFINITE, "mp_field_load: non-finite face flow"));
+    if (got.flags & 2u) return fin(fail(MP_ERR_NONFINITE, "mp_field_load: porosity outside (0, 1] in an active cell"));
+    if (got.flags & 4u) return fin(fail(MP_ERR_INVALID_ARG, "mp_field_load: ibound outside {-1, 0, 1, 2}"));
+    mp_balance bal{};
+    if ((e = balance_report(ctx, got.total, dio, ncell, parts, &bal)) != cudaSuccess)
+        return fin(cuda_fail(e, "mp_field_load: balance"));
+    cudaFreeAsync(stage, s);
 
     mp_field* f = new mp_field();
     f->ctx = ctx;
-    f->d.nlay = (int)nl; f->d.nrow = (int)nr; f->d.ncol = (int)nc;
-    f->d.ncell = ncell;
-    f->d.rec64 = reinterpret_cast<CellF64*>(buf + o_r64);
-    f->d.rec32 = reinterpret_cast<CellF32*>(buf + o_r32);
-    f->d.delr = reinterpret_cast<double*>(buf + o_delr);
-    f->d.delc = reinterpret_cast<double*>(buf + o_delc);
-    f->d.dz = reinterpret_cast<double*>(buf + o_dz);
-    f->d.ax = reinterpret_cast<AxisCell*>(buf + o_ax);
-    f->d.no_screen = no_screen;
-    f->d.xf = reinterpret_cast<double*>(buf + o_xf);
-    f->d.yf = reinterpret_cast<double*>(buf + o_yf);
-    f->d.zf = reinterpret_cast<double*>(buf + o_zf);
-    f->d.ibound = reinterpret_cast<int8_t*>(buf + o_ib);
-    f->d.sinkfrac = reinterpret_cast<double*>(buf + o_sf);
-    f->d.m_ncol = div_magic((unsigned)nc);
-    f->d.m_nrow = div_magic((unsigned)nr);
-    double2* dio = nullptr;
-    e = cudaMalloc(&dio, sizeof(double2) * (size_t)std::max(ncell, 1LL));
-    if (e == cudaSuccess)
-        e = launch_build_records(f->d, const_cast<CellF64*>(f->d.rec64), const_cast<CellF32*>(f->d.rec32),
-                                 reinterpret_cast<double*>(buf + o_sf), dio, qx, qy, qz, por, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaStreamDestroy(s);
-    if (stage) cudaFree(stage);
-    if (e == cudaSuccess) {
-        // the balance report (ibound on the host: the caller's array, or a copy)
-        std::vector<int8_t> hib;
-        const int8_t* ibh = d->ibound;
-        if (dev_in) {
-            hib.resize((size_t)ncell);
-            e = cudaMemcpy(hib.data(), buf + o_ib, (size_t)ncell, cudaMemcpyDeviceToHost);
-            ibh = hib.data();
-        }
-        if (e == cudaSuccess && balance_from_device(dio, ibh, ncell, &f->balance) != MP_OK) e = cudaErrorUnknown;
-    }
-    if (dio) cudaFree(dio);
-    if (e != cudaSuccess) {
-        delete f;
-        cudaFree(buf);
-        return cuda_fail(e, "mp_field_load: build records");
-    }
+    f->d = v;
+    f->balance = bal;
     f->buf = buf;
     f->bytes = persistent;
     f->geom.reserve(6 + nc + nr + nl);
@@ -466,12 +477,15 @@ int mp_field_free(mp_field* f)
     mp_ctx* ctx = f->ctx;
     int rc = drain_users(ctx, nullptr, f);
     if (rc != MP_OK) return rc;
+    // every stream's work first (a release or an allocation-free launch may
+    // still read the field): the memory is handed on in load_st's order
+    cudaSetDevice(ctx->device);
+    MP_CUDA(cudaDeviceSynchronize(), "mp_field_free");
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
         ctx->fields.erase(f);
     }
-    cudaSetDevice(ctx->device);
-    cudaFree(f->buf);
+    cudaFreeAsync(f->buf, ctx->load_st);
     delete f;
     return MP_OK;
 }
@@ -516,11 +530,18 @@ int mp_usg_field_load(mp_ctx* ctx, const mp_usg_desc* d, mp_field** out)
     const size_t o_ib = off; off = align256(off + (size_t)nc);
     const size_t o_sf = off; off = align256(off + sizeof(double) * (size_t)nc);
     const size_t persistent = off;
-    const size_t o_box = off; off = align256(off + sizeof(double) * 6 * (size_t)nc);
-    const size_t o_por = off; off = align256(off + sizeof(double) * (size_t)nc);
+    size_t soff = 0;   // scratch, freed once the records are built
+    const size_t o_box = soff; soff = align256(soff + sizeof(double) * 6 * (size_t)nc);
+    const size_t o_por = soff; soff = align256(soff + sizeof(double) * (size_t)nc);
+    const size_t o_io = soff; soff = align256(soff + sizeof(double2) * (size_t)nc);
+    const size_t o_part = soff; soff = align256(soff + sizeof(BalancePart) * (BALANCE_BLOCKS + 1));
+    const cudaStream_t s = ctx->load_st;
     char* buf = nullptr;
-    if (cudaMalloc(&buf, off) != cudaSuccess) {
+    char* stage = nullptr;
+    if (cudaMallocFromPoolAsync(&buf, persistent, ctx->field_pool, s) != cudaSuccess ||
+        cudaMallocFromPoolAsync(&stage, soff, ctx->field_pool, s) != cudaSuccess) {
         cudaGetLastError();
+        if (buf) cudaFreeAsync(buf, s);
         return fail(MP_ERR_OOM, "mp_usg_field_load: device allocation failed");
     }
     std::vector<mp::UsgSub> sub((size_t)std::max(ns, 1LL));
@@ -540,24 +561,28 @@ int mp_usg_field_load(mp_ctx* ctx, const mp_usg_desc* d, mp_field** out)
     u.sub = reinterpret_cast<mp::UsgSub*>(buf + o_sub);
     u.ibound = reinterpret_cast<int8_t*>(buf + o_ib);
     u.sinkfrac = reinterpret_cast<double*>(buf + o_sf);
-    cudaError_t e = cudaMemcpy(buf + o_fo, d->face_off, sizeof(long long) * (size_t)(6 * nc + 1),
-                               cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(buf + o_sub, sub.data(), sizeof(mp::UsgSub) * sub.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(buf + o_ib, d->ibound, (size_t)nc, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(buf + o_box, d->box, sizeof(double) * 6 * (size_t)nc, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(buf + o_por, d->porosity, sizeof(double) * (size_t)nc, cudaMemcpyHostToDevice);
-    double2* dio = nullptr;
-    if (e == cudaSuccess) e = cudaMalloc(&dio, sizeof(double2) * (size_t)std::max(nc, 1LL));
+    const cudaMemcpyKind h2d = cudaMemcpyHostToDevice;
+    cudaError_t e = cudaMemcpyAsync(buf + o_fo, d->face_off, sizeof(long long) * (size_t)(6 * nc + 1), h2d, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(buf + o_sub, sub.data(), sizeof(mp::UsgSub) * sub.size(), h2d, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(buf + o_ib, d->ibound, (size_t)nc, h2d, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(stage + o_box, d->box, sizeof(double) * 6 * (size_t)nc, h2d, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(stage + o_por, d->porosity, sizeof(double) * (size_t)nc, h2d, s);
+    double2* dio = reinterpret_cast<double2*>(stage + o_io);
+    BalancePart* parts = reinterpret_cast<BalancePart*>(stage + o_part);
+    BalancePart total{};
     if (e == cudaSuccess)
         e = mp::launch_build_usg(u, const_cast<mp::UsgCell*>(u.cell), const_cast<mp::UsgGeo*>(u.geo),
-                                 reinterpret_cast<double*>(buf + o_sf), dio, reinterpret_cast<double*>(buf + o_box),
-                                 reinterpret_cast<double*>(buf + o_por), nullptr);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+                                 reinterpret_cast<double*>(buf + o_sf), dio, reinterpret_cast<double*>(stage + o_box),
+                                 reinterpret_cast<double*>(stage + o_por), s);
+    if (e == cudaSuccess) e = launch_balance(dio, u.ibound, nc, parts, parts + BALANCE_BLOCKS, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&total, parts + BALANCE_BLOCKS, sizeof(total), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     mp_balance bal{};
-    if (e == cudaSuccess && balance_from_device(dio, d->ibound, nc, &bal) != MP_OK) e = cudaErrorUnknown;
-    if (dio) cudaFree(dio);
+    if (e == cudaSuccess) e = balance_report(ctx, total, dio, nc, parts, &bal);
+    cudaFreeAsync(stage, s);
     if (e != cudaSuccess) {
-        cudaFree(buf);
+        cudaFreeAsync(buf, s);
+        cudaStreamSynchronize(s);
         return cuda_fail(e, "mp_usg_field_load");
     }
     mp_field* f = new mp_field();

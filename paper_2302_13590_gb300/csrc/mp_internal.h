@@ -216,6 +216,24 @@ inline void split_ff(double v, float& hi, float& lo)
     lo = (v - (double)hi < 3.0e38 && v - (double)hi > -3.0e38) ? (float)(v - (double)hi) : 0.0f;
 }
 
+// Volume balance of a field, reduced on the device.
+struct BalancePart {
+    double max_abs;      // largest residual of the active cells (NaN apart); cell: the first with it, -1: none
+    double max_rel;
+    double r_first;      // residual of the first active cell (first: its index, -1: none)
+    long long cell;
+    long long first;
+    long long active;
+    long long sinks;
+};
+constexpr int BALANCE_BLOCKS = 1024;   // parts: [BALANCE_BLOCKS]
+// inout is overwritten: the sink cells' extractions stay in it, block by block
+cudaError_t launch_balance(double2* inout, const int8_t* ibound, long long ncell, BalancePart* parts,
+                           BalancePart* total, cudaStream_t s);
+// the extractions that launch_balance left, packed in cell order
+cudaError_t launch_balance_sinks(const double2* inout, long long ncell, const BalancePart* parts, double* sinks,
+                                 cudaStream_t s);
+
 // Kernel launchers (each enqueues one kernel on `s`).
 cudaError_t launch_validate(const double* qx, long long nqx, const double* qy, long long nqy, const double* qz,
                             long long nqz, const double* por, const int8_t* ib, long long ncell, unsigned* flags,
