@@ -202,6 +202,24 @@ __device__ __forceinline__ double f2d_normal_pos(float f)
     return __hiloint2double((int)((fb >> 3) + 0x38000000u), (int)(fb << 29));
 }
 
+// 1 / x rounded to nearest for normal x with a normal reciprocal: the
+// hardware's approximation and one Newton step in fmas, which rounds
+// correctly (P. W. Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM J. Res. Dev. 34(1), 1990), compared with
+// __frcp_rn over every significand (tests/cuda/f64_fast_check.cu); the
+// general function takes 200 cycles of latency, this about 40
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_rn_normal(float x)
+{
+    const float y = rcp_approx(x);
+    return __fmaf_rn(y, __fmaf_rn(-x, y, 1.0f), y);
+}
+
 // d / v as d times 1 / v: the IEEE FP32 reciprocal y0 of the truncated v
 // (relative error below 1.8e-7), then one third-order step
 // y = y0 + y0 (e + e^2) with e = 1 - v y0 in one fma (rounded by less
@@ -216,7 +234,7 @@ __device__ __forceinline__ double f64_div(double d, double v)
     unsigned lo, hi;
     words(v, lo, hi);
     if (hi_abs(hi) - 0x38700000u >= 0x0f100000u) return div_ieee(d, v);   // 2^-120 <= |v| < 2^121
-    const double y0 = f2d_normal(__frcp_rn(trunc_normal(lo, hi)));   // |1 / v| in (2^-121, 2^120]: normal
+    const double y0 = f2d_normal(rcp_rn_normal(trunc_normal(lo, hi)));   // |1 / v| in (2^-121, 2^120]: normal
     const double e0 = fma(-v, y0, 1.0);
     const double y1 = fma(y0, fma(e0, e0, e0), y0);
     return d * y1;
@@ -423,15 +441,18 @@ __device__ __forceinline__ double series_expm1(double w)
 
 // Exit time along one axis from the distance d to its reachable face at the
 // particle velocity vp: t1 = d / vp by f64_div, z = A t1, t1 when z == 0,
-// else log1p(z) * (1 / A).
-__device__ __forceinline__ double f64_exit_time_d(double A, double iA, double d, double vp)
+// else log1p(z) * (1 / A).  (A z that is not used is replaced by one inside a
+// row of log1p's table, so that it does not send the warp to the FP64 sum; so
+// is that of a lane without use, whose result means nothing.)
+__device__ __forceinline__ double f64_exit_time_d(double A, double iA, double d, double vp, bool use = true)
 {
     const double t1 = f64_div(d, vp);
     const double z = A * t1;
-    const double te = fast_log1p(z) * iA;
     unsigned lo, hi;
     words(z, lo, hi);
-    return zero_w(lo, hi) ? t1 : te;
+    const bool lin = zero_w(lo, hi);
+    const double te = fast_log1p(lin || !use ? 0.7 : z) * iA;
+    return lin ? t1 : te;
 }
 
 // the reachable face (+1, -1, 0: none) from the words of vp and the signs of
@@ -513,12 +534,6 @@ __device__ __forceinline__ double f64_move_fast(double A, double iA, double D, d
 // carries the information there): below 4.6e-5, since |ln u| >= 0.0078
 // wherever the logarithm is used.  In all below 1.2e-4, a quarter of the
 // 2^-11 that the candidate margin of 2^-10 allows.
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float lg2_approx(float x)
 {
     float y;

@@ -1,8 +1,8 @@
 // Checks the FP64 step's short forms (mp_f64math.cuh) against the general
 // ones, bit for bit: fast_log1p against series_log1p (around every row edge,
 // sqrt2 and the ends of the table too), f64_move_fast against f64_move, the
-// word forms of the FP32 truncation against f32_trunc, the time keys against
-// the FP64 order, and the screened exit axis against all three exact times.
+// word forms of the FP32 truncation against f32_trunc, the FP32 reciprocal
+// against __frcp_rn on every significand, the time keys against the FP64 order, and the screened exit axis against all three exact times.
 // Prints the mismatch counts and exits non-zero on any.
 #include <cstdio>
 
@@ -81,6 +81,11 @@ __global__ void check(unsigned long long* bad, unsigned long long n)
         if (__float_as_uint(trunc_small(lo, hi)) != want) atomicAdd(bad + 2, 1ULL);
         if (t > 0.0 && __float_as_uint(trunc_pos(lo, hi)) != want) atomicAdd(bad + 2, 1ULL);
         if (fabs(t) >= 0x1.0p-126 && __float_as_uint(trunc_normal(lo, hi)) != want) atomicAdd(bad + 2, 1ULL);
+        // the FP32 reciprocal: every significand, both signs, exponents over
+        // the range that d / v takes
+        const float rx = __uint_as_float((unsigned)(i & 0x7fffffu) | ((7u + (unsigned)(mix64(i >> 23) % 240)) << 23) |
+                                         ((unsigned)(r >> 40) << 31));
+        if (__float_as_uint(rcp_rn_normal(rx)) != __float_as_uint(__frcp_rn(rx))) atomicAdd(bad + 6, 1ULL);
         // keys of times
         const double a = (c & 8 ? 1.0 : -1.0) * spread(mix64(r + 7), -3, 3) * (c % 23 == 0 ? 0.0 : 1.0) + 0.0;
         const double b = c % 29 == 0 ? a : (c & 16 ? 1.0 : -1.0) * spread(mix64(r + 8), -3, 3) * (c % 31 == 0 ? 0.0 : 1.0);
@@ -146,8 +151,8 @@ int main()
     unsigned long long h[8] = {0};
     cudaMemcpy(h, bad, sizeof h, cudaMemcpyDeviceToHost);
     const cudaError_t e = cudaDeviceSynchronize();
-    printf("%s log1p %llu move %llu trunc %llu keys %llu face %llu screen %llu\n", cudaGetErrorString(e), h[0], h[1],
-           h[2], h[3], h[4], h[5]);
+    printf("%s log1p %llu move %llu trunc %llu keys %llu face %llu screen %llu rcp %llu\n", cudaGetErrorString(e),
+           h[0], h[1], h[2], h[3], h[4], h[5], h[6]);
     cudaFree(bad);
-    return (e == cudaSuccess && !(h[0] | h[1] | h[2] | h[3] | h[4] | h[5])) ? 0 : 1;
+    return (e == cudaSuccess && !(h[0] | h[1] | h[2] | h[3] | h[4] | h[5] | h[6])) ? 0 : 1;
 }
