@@ -869,6 +869,250 @@ struct F64Engine {
     }
 };
 
+// ---------------------------------------------------------------------------
+// few particles: three lanes a particle
+// ---------------------------------------------------------------------------
+
+// What bounds a step here: a FP64 instruction occupies its SM sub-partition
+// for 64 cycles whatever its active lanes, and one warp cannot overlap two of
+// them (measured: two independent chains of fmas take twice one chain's time).
+// So while there are no more warps than a few a sub-partition, a step takes
+// its FP64 warp instructions and the integer code between them, and lanes are
+// free.  Lane 3 g + a of a warp holds axis a of the warp's particle g:
+// velocities, exit times and motions of the axes run in the same
+// instructions, 27 FP64 ones a step instead of 37.  The axes agree on the
+// smallest FP32 estimate (so that a lane that cannot win never sends the warp
+// into log1p's general form), then on the smallest exact time, by shuffles;
+// the next cell's record is read while the axes move; and everything but
+// crossing into the next cell is one rare branch, run on the group's first
+// lane with the axes gathered through the one-lane engine's own functions.
+// Every particle has its lanes from the start, so the schedules would give
+// the same.  One step of 4864 particles 2.7 -> 1.7 us; 1000 particles, 50x50
+// cells 135 -> 93 us; 5003 pathlines, 7x61x83 cells 449 -> 277 us; 10,000
+// particles to a stop time, 200x200x20 cells 772 -> 491 us.
+constexpr int AXES_PARTICLES = 10;   // a warp (30 of its lanes)
+// Launches of up to this many particles take three lanes each: 12 warps an SM
+// (three a sub-partition) on 152 SMs.  There both forms are FP64 bound at
+// about the same time (endpoints, 200x200x20 cells, 329 steps the longest:
+// 4864 particles 550 us against 880, 9728: 629 / 947, 19456: 1020 / 979,
+// 38912: 2317 / 1050).
+constexpr long long AXES_MAX = 12 * 152 * AXES_PARTICLES;
+
+// one axis of a cell's record
+struct AxisRec {
+    double v1, A, iA, D;
+    float f1, f2, fA;
+    unsigned nb;
+};
+__device__ __forceinline__ AxisRec read_axis(const DevField& f, int c, int a, int at)
+{
+    const double* rp = reinterpret_cast<const double*>(f.rec64 + c);
+    const float* fp = reinterpret_cast<const float*>(rp + 10) + 3 * a;
+    return AxisRec{__ldg(rp + 3 * a), __ldg(rp + 3 * a + 1), __ldg(rp + 3 * a + 2), __ldg(&f.ax[at].D),
+                   __ldg(fp), __ldg(fp + 1), __ldg(fp + 2), __ldg(reinterpret_cast<const unsigned*>(rp + 9))};
+}
+
+// the full position and cell indices of each particle on its three lanes
+// (warp-uniform call)
+template <class S>
+__device__ __forceinline__ void gather_axes(S& s, double x, int ix, int base)
+{
+    const unsigned FULL = 0xffffffffu;
+    s.x0 = __shfl_sync(FULL, x, base);
+    s.x1 = __shfl_sync(FULL, x, base + 1);
+    s.x2 = __shfl_sync(FULL, x, base + 2);
+    s.j = __shfl_sync(FULL, ix, base);
+    s.i = __shfl_sync(FULL, ix, base + 1);
+    s.k = __shfl_sync(FULL, ix, base + 2);
+}
+
+template <bool ONE, bool TS, bool PL>
+__global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
+{
+    using E = F64Engine<ONE>;
+    const DevField& f = e.f;
+    __shared__ unsigned long long s_cnt[N_COUNTERS];
+    typename E::RecQ& Q = *reinterpret_cast<typename E::RecQ*>(s_dyn);
+    PathQ& P = *reinterpret_cast<PathQ*>(s_dyn + (TS ? sizeof(typename E::RecQ) : 0));
+    if (threadIdx.x < N_COUNTERS) s_cnt[threadIdx.x] = 0ULL;
+    window_begin(e);
+    __syncwarp();
+    const unsigned FULL = 0xffffffffu;
+    // (lanes 30 and 31 hold no particle: they follow the first group's shuffles)
+    const int lane = threadIdx.x & 31, grp = lane / 3, a = lane - 3 * grp, base = grp < AXES_PARTICLES ? 3 * grp : 0;
+    const bool lead = a == 0;
+    const int stride_y = f.ncol, stride_z = f.ncol * f.nrow;
+    const int axis_at = a == 0 ? 0 : (a == 1 ? f.ncol : f.ncol + f.nrow);
+    int qcount = 0, pcount = 0;
+    long long q = 0;
+    typename E::State s;   // x0, x1, x2, i, j, k: as last gathered
+    s.r = 0;
+    s.steps = 0;
+    s.st = ST_SKIP;
+    s.c = -1;
+    s.x0 = s.x1 = s.x2 = 0.0;
+    s.i = s.j = s.k = 0;
+    bool live = false, ended = false, loaded = false;
+    const long long g = (long long)blockIdx.x * AXES_PARTICLES + grp;
+    if (grp < AXES_PARTICLES && g < e.b.n_total) {
+        const int r = request_of(e, g, q);
+        e.template load<TS>(r, q, s);
+        live = s.st == MP_ST_ACTIVE;
+        ended = !live && s.st != ST_SKIP;
+        loaded = true;
+    }
+    if (PL)
+        pl_push(e, P, pcount, s, q, lead && loaded && path_start(e, s), s.st == MP_ST_TIME ? MP_ST_ACTIVE : s.st);
+    if (TS) tail_fill(e, s, q, lead && ended && !paused(e, s));
+    if (lead && ended) e.template finish<TS>(q, s, s_cnt);
+    // this lane's axis: offset and index, and the cell's record of it
+    double x = a == 0 ? s.x0 : (a == 1 ? s.x1 : s.x2);
+    int ix = a == 0 ? s.j : (a == 1 ? s.i : s.k);
+    AxisRec c{};
+    c.D = 1.0;
+    if (live) c = read_axis(f, s.c, a, axis_at + ix);
+    const int next1 = base + (a == 2 ? 0 : a + 1), next2 = base + (a == 0 ? 2 : a - 1);
+    bool exact = false;   // every reachable axis in this step
+    bool going = __any_sync(FULL, live);
+    while (going) {
+        const TrackParams& p = e.req(s.r).p;
+        const bool go = live && !(s.steps >= s.cap && (long long)s.steps >= p.max_steps);
+        // velocity, reachable face, FP32 estimate of the time to it (as in
+        // the one-lane engine; -1: not to be trusted)
+        const double vp = f64_vel(c.v1, c.A, x);
+        unsigned lo, hi;
+        words(vp, lo, hi);
+        const int face = go ? f64_face(lo, hi, c.nb >> (NB_SIGN + 4 * a)) : 0;
+        const unsigned up = __ballot_sync(FULL, face > 0);
+        const double d = f64_face_dist(face, c.D, x);
+        float est = CUDART_INF_F;
+        if (face) {
+            unsigned dl, dh;
+            words(d, dl, dh);
+            est = f32_estimate(trunc_small(dl, dh), trunc_normal(lo, hi), c.fA, face > 0 ? c.f2 : c.f1);
+            if (!(est < CUDART_INF_F) || !vel_trusted(hi) || f.no_screen) est = -1.0f;
+        }
+        const float em = fminf(est, fminf(__shfl_sync(FULL, est, next1), __shfl_sync(FULL, est, next2)));
+        // the exact time of the axes within 2^-10 of the smallest estimate
+        // (all reachable ones in doubt); the smallest wins, ties to the lower axis
+        const bool use = face != 0 && (exact || em < 0.0f || est <= em * (1.0f + 0.0009765625f));
+        const double te = f64_exit_time_d(c.A, c.iA, d, face ? vp : 1.0, use);
+        words(te, lo, hi);
+        const bool has = use && hi_abs(hi) < 0x7ff00000u;
+        const unsigned long long key = has ? (unsigned long long)hi_abs(hi) << 32 | lo : 0x7ff0000000000000ULL;
+        const unsigned long long k0 = __shfl_sync(FULL, key, base), k1 = __shfl_sync(FULL, key, base + 1),
+                                 k2 = __shfl_sync(FULL, key, base + 2);
+        int ax = -1;
+        unsigned long long km = 0x7ff0000000000000ULL;
+        if (k0 < km) { km = k0; ax = 0; }
+        if (k1 < km) { km = k1; ax = 1; }
+        if (k2 < km) { km = k2; ax = 2; }
+        const double tmin = __longlong_as_double((long long)km);
+        const int fx = ax < 0 ? 0 : ((up >> (base + ax)) & 1u) ? 1 : -1;
+        const int fidx = 2 * ax + (fx > 0 ? 1 : 0);
+        // the neighbour across the exit face, read while the axes move
+        const int cls = ax < 0 ? (int)NB_OUTSIDE : (int)((c.nb >> (2 * fidx)) & 3u);
+        const int c2 = s.c + fx * (ax == 0 ? 1 : (ax == 1 ? stride_y : stride_z));
+        const int ix2 = ix + (a == ax ? fx : 0);
+        const bool enter = go && ax >= 0 && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
+        AxisRec n = c;
+        if (enter) n = read_axis(f, c2, a, axis_at + ix2);
+        const double t_end = s.t + tmin;
+        bool again;
+        double xn = f64_move_fast(c.A, c.iA, c.D, vp, x, tmin, again);
+        again = again && a != ax;
+        // an event: an output time or the stop time in the step, no exit, a
+        // path that ends here, the step cap, a motion for the general form
+        const bool ev = go && (ax < 0 || tkey(t_end) >= s.tev);
+        if (__any_sync(FULL, ev || (live && (!go || !enter || again)))) {
+            if (__any_sync(FULL, go && !exact && ax < 0 && face != 0)) {   // the leading time was not usable
+                exact = true;
+                continue;
+            }
+            enum { P_NONE, P_CROSS, P_TIME, P_NOEXIT, P_CAPTURE };
+            int path = go ? P_CROSS : P_NONE, m = 0;
+            if (ev) {   // (the stop time is never before tev)
+                if (ax < 0 && s.in_sink) path = P_CAPTURE;
+                else if (ax < 0 && !(p.t_stop < CUDART_INF)) path = P_NOEXIT;
+                else if (ax < 0 || ge_d(t_end, p.t_stop)) path = P_TIME;
+                if (TS && path != P_CAPTURE) {
+                    const DevOut& o = e.req(s.r).o;
+                    const double t_rec = path == P_NOEXIT ? CUDART_INF : (path == P_TIME ? p.t_stop : t_end);
+                    int kk = s.kn;
+                    while (kk < p.n_times && ge_d(t_rec, __ldg(o.times + kk))) kk++;
+                    m = kk - s.kn;
+                }
+            }
+            if (TS && __any_sync(FULL, m > 0)) {
+                gather_axes(s, x, ix, base);
+                rq_push(e, Q, qcount, s, q, s.kn, lead ? m : 0, path == P_NOEXIT ? MP_ST_NO_EXIT : MP_ST_ACTIVE);
+                if (m) {
+                    s.kn += m;
+                    s.tev = e.next_event(s);
+                }
+            }
+            if (path == P_CROSS) {
+                if (again) xn = f64_move(c.A, c.iA, c.D, vp, x, tmin);
+                if (!enter) {
+                    x = a == ax ? (fx > 0 ? c.D : 0.0) : xn;
+                    s.t = t_end;
+                    s.ef = fidx;
+                    s.st = cls == NB_OUTSIDE ? MP_ST_EXIT_DOMAIN : (cls == NB_BOUNDARY ? MP_ST_BOUNDARY : MP_ST_SINK);
+                }
+            } else if (path == P_TIME) {
+                x = f64_move(c.A, c.iA, c.D, vp, x, p.t_stop - s.t);
+                s.t = p.t_stop;
+                s.st = MP_ST_TIME;
+            } else if (live) {
+                s.st = path == P_CAPTURE ? MP_ST_SINK : (path == P_NOEXIT ? MP_ST_NO_EXIT : MP_ST_STEP_CAP);
+            }
+            ended = live && s.st != MP_ST_ACTIVE;
+            if (__any_sync(FULL, ended)) {
+                if (go && ended) s.steps++;
+                gather_axes(s, x, ix, base);
+                if (PL) pl_push(e, P, pcount, s, q, lead && go && ended && p.pathline, s.st);
+                if (TS) tail_fill(e, s, q, lead && ended && !paused(e, s));
+                if (ended && lead) e.template finish<TS>(q, s, s_cnt);
+                live = live && !ended;
+                going = __any_sync(FULL, live);
+            }
+        }
+        exact = false;
+        if (go && live) {
+            // hand over to the neighbour; the exit coordinate enters on the shared face
+            s.steps++;
+            x = a == ax ? (fx < 0 ? n.D : 0.0) : xn;
+            s.t = t_end;
+            s.ef = fidx;
+            s.in_sink = cls == NB_SINK;
+            s.c = c2;
+            ix = ix2;
+            s.h = fnv_step(s.h, c2);
+            c = n;
+        }
+        if (PL) {
+            gather_axes(s, x, ix, base);
+            pl_push(e, P, pcount, s, q, lead && go && live && p.pathline, s.st);
+        }
+    }
+    if (TS) rq_drain(e, Q, qcount, true);
+    if (PL) pl_flush(e, P, pcount);
+    flush_counters(e, s_cnt);
+    window_end(e);
+}
+
+template <bool ONE>
+cudaError_t launch_axes(const F64Engine<ONE>& e, unsigned modes, cudaStream_t s)
+{
+    const bool ts = (modes & MODE_TS) != 0, pl = (modes & MODE_PATH) != 0;
+    const size_t smem = (ts ? sizeof(typename F64Engine<ONE>::RecQ) : 0) + (pl ? sizeof(PathQ) : 0);
+    const unsigned grid = (unsigned)((e.b.n_total + AXES_PARTICLES - 1) / AXES_PARTICLES);
+    auto kern = ts ? (pl ? k_track_axes<ONE, true, true> : k_track_axes<ONE, true, false>)
+                   : (pl ? k_track_axes<ONE, false, true> : k_track_axes<ONE, false, false>);
+    kern<<<grid, 32, smem, s>>>(e);
+    return cudaGetLastError();
+}
+
 // A request's endpoint arrays into the caller's: one launch for up to twelve
 // copies (blockIdx.y) instead of a cudaMemcpyAsync each, which cost 34 us of
 // host time and about 2 us of stream time apiece for 1000 particles.  Bound
@@ -950,8 +1194,14 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s)
 cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
                               int blocks_per_sm_cap, cudaStream_t s)
 {
-    if (b.n_reqs == 1) return launch_tracking(F64Engine<true>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
-    return launch_tracking(F64Engine<false>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_total <= 0) return cudaSuccess;
+    const bool few = b.n_total <= AXES_MAX;
+    if (b.n_reqs == 1) {
+        const F64Engine<true> e{f, b};
+        return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    }
+    const F64Engine<false> e{f, b};
+    return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
 }
 
 }  // namespace mp
