@@ -443,6 +443,7 @@ cudaError_t launch_release_explicit(const DevField& f, const DevState& st, long 
 template <bool ONE_REQ>
 struct F64Engine {
     static constexpr bool ONE = ONE_REQ;
+    static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
     // blocks of 256 threads to keep resident per SM (0: no target; the
     // kernels are FP64-pipe bound)
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
@@ -1095,7 +1096,7 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
             pl_push(e, P, pcount, s, q, lead && go && live && p.pathline, s.st);
         }
     }
-    if (TS) rq_drain(e, Q, qcount, true);
+    if (TS) rec_finish(e, Q, qcount);
     if (PL) pl_flush(e, P, pcount);
     flush_counters(e, s_cnt);
     window_end(e);

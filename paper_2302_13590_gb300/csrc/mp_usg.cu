@@ -146,6 +146,7 @@ cudaError_t launch_release_explicit_usg(const DevUsg& u, const DevState& st, lon
 template <bool ONE_REQ>
 struct UsgEngine {
     static constexpr bool ONE = ONE_REQ;
+    static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevUsg u;
     Batch b;
