@@ -585,7 +585,7 @@ struct F64Engine {
     }
 
     // per-warp queue of deferred timeseries records (structure of arrays)
-    struct RecQ {
+    struct alignas(16) RecQ {
         double p0[RQ_CAP], p1[RQ_CAP], p2[RQ_CAP], t[RQ_CAP];
         long long q[RQ_CAP];
         int c[RQ_CAP], i[RQ_CAP], j[RQ_CAP], k[RQ_CAP], kk[RQ_CAP], st[RQ_CAP], r[RQ_CAP];

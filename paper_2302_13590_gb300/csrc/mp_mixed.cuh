@@ -298,7 +298,7 @@ struct MixEngine {
     // deferred timeseries records: REC_SLOTS of each lane (slot 32 k + lane),
     // kept small, since what the block's queues take of the SM's shared
     // memory its L1 does not have for the field's records
-    struct RecQ {
+    struct alignas(16) RecQ {
         static constexpr int N = 32 * REC_SLOTS;
         float x0[N], x1[N], x2[N], tau[N];
         int c[N];

@@ -243,7 +243,7 @@ __device__ __forceinline__ void tail_fill(const E& e, const typename E::State& s
 
 constexpr int PQ_CAP = 64;   // points per warp queue (>= 2 x 32)
 
-struct PathQ {
+struct alignas(16) PathQ {
     double x[PQ_CAP], y[PQ_CAP], z[PQ_CAP], t[PQ_CAP];
     int q[PQ_CAP], c[PQ_CAP], r[PQ_CAP];
     unsigned seq[PQ_CAP];
@@ -438,6 +438,10 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
 
 // One variant of the tracking kernel: opt in to more than 48 KB of dynamic
 // shared memory when the queues need it, size a persistent grid by occupancy.
+// (the queues of a block follow one another in dynamic shared memory: each
+// size keeps the next one's doubles aligned)
+static_assert(sizeof(PathQ) % 16 == 0, "queue sizes are whole 16-byte words");
+
 template <class E, bool TS, bool PL>
 cudaError_t launch_variant(const E& e, int schedule, int block, int blocks_per_sm_cap, size_t smem, cudaStream_t st)
 {

@@ -255,7 +255,7 @@ struct UsgEngine {
         s.tev = TS ? next_event(s) : bound_key(p.t_stop);
     }
 
-    struct RecQ {
+    struct alignas(16) RecQ {
         double p0[RQ_CAP], p1[RQ_CAP], p2[RQ_CAP], tau[RQ_CAP];
         long long q[RQ_CAP];
         int c[RQ_CAP], kk[RQ_CAP], st[RQ_CAP], r[RQ_CAP];
