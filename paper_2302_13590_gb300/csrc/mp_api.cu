@@ -892,7 +892,6 @@ int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream
     p.t_stop = t_stop;
     p.max_steps = o->max_steps > 0 ? o->max_steps : 1000000LL;
     p.n_times = nt;
-    p.steps_per_fetch = o->steps_per_fetch > 0 ? o->steps_per_fetch : 4;
     p.update_group = (o->flags & MP_TRACK_UPDATE_GROUP) ? 1 : 0;
     p.pass_sinks = (o->flags & MP_TRACK_PASS_WEAK_SINKS) ? 1 : 0;
     p.sink_frac = o->weak_sink_fraction;
@@ -931,7 +930,7 @@ int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, const
 {
     mp::Batch b{};
     b.n_reqs = n;
-    b.steps_per_fetch = spf > 0 ? spf : 4;
+    b.steps_per_fetch = spf;
     char* tbl = nullptr;
     cudaError_t e = cudaSuccess;
     if (n == 1) {
@@ -1002,7 +1001,7 @@ void resolve_launch(mp_ctx* ctx, const mp_field* f, int precision, bool ts, cons
     if (*sched != MP_SCHED_AUTO) return;
     *sched = MP_SCHED_DYNAMIC;
     *blk = 128;
-    *spf = 4;
+    *spf = 0;
     std::lock_guard<std::mutex> lk(ctx->mu);
     auto it = ctx->tuned.find(TuneKey{f, precision, ts ? 1 : 0});
     if (it != ctx->tuned.end()) {
@@ -1766,7 +1765,7 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
         const int prec = p == 0 ? MP_PREC_FP64 : MP_PREC_MIXED;
         int sched = 0, blk = 0, spf = 0;
         resolve_launch(ctx, f, prec, (modes[p] & mp::MODE_TS) != 0, opts[sel[p][0]], &sched, &blk, &spf);
-        bat[p].steps_per_fetch = spf > 0 ? spf : 4;
+        bat[p].steps_per_fetch = spf;
         e = prec == MP_PREC_FP64 ? mp::launch_track_fp64(fd, bat[p], modes[p], sched, blk > 0 ? blk : 128, 0, cs)
                                  : mp::launch_track_mixed(fd, bat[p], modes[p], sched, blk > 0 ? blk : 128, 0, cs);
         if (e == cudaSuccess) e = mp::launch_spread_window(bat[p], cs);

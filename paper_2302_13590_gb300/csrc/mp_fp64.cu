@@ -444,6 +444,7 @@ template <bool ONE_REQ>
 struct F64Engine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
+    static constexpr int FETCH = 4;            // steps per fetch
     // blocks of 256 threads to keep resident per SM (0: no target; the
     // kernels are FP64-pipe bound)
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
@@ -891,7 +892,6 @@ struct F64Engine {
 // the same.  One step of 4864 particles 2.7 -> 1.7 us; 1000 particles, 50x50
 // cells 135 -> 93 us; 5003 pathlines, 7x61x83 cells 449 -> 277 us; 10,000
 // particles to a stop time, 200x200x20 cells 772 -> 491 us.
-constexpr int AXES_PARTICLES = 10;   // a warp (30 of its lanes)
 // Launches of up to this many particles take three lanes each: 12 warps an SM
 // (three a sub-partition) on 152 SMs.  There both forms are FP64 bound at
 // about the same time (endpoints, 200x200x20 cells, 329 steps the longest:

@@ -168,7 +168,6 @@ struct TrackParams {
     double t_stop;
     long long max_steps;
     int n_times;
-    int steps_per_fetch;
     int update_group;
     int pass_sinks;              // enter sink cells, leave through outflow faces
     double sink_frac;            // > 0 with pass_sinks: sinks extracting at least this fraction still stop
@@ -205,7 +204,7 @@ struct Batch {
     const long long* starts;     // n_reqs > 1: [n_reqs + 1], device
     int n_reqs;
     long long n_total;
-    int steps_per_fetch;
+    int steps_per_fetch;         // dynamic schedule; <= 0: chosen at launch
     unsigned long long* queue;   // dynamic schedule head (zeroed before launch)
 };
 

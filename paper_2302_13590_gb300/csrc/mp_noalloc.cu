@@ -128,7 +128,6 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     p.t_stop = (want_ts && !(o->mode & MP_MODE_ENDPOINT) && !(o->t_stop < INFINITY)) ? o->times[nt - 1] : o->t_stop;
     p.max_steps = o->max_steps > 0 ? o->max_steps : 1000000LL;
     p.n_times = nt;
-    p.steps_per_fetch = o->steps_per_fetch > 0 ? o->steps_per_fetch : 4;
     p.update_group = (o->flags & MP_TRACK_UPDATE_GROUP) ? 1 : 0;
     p.pass_sinks = (o->flags & MP_TRACK_PASS_WEAK_SINKS) ? 1 : 0;
     p.sink_frac = o->weak_sink_fraction;
@@ -143,7 +142,7 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     b.one.p = p;
     b.n_reqs = 1;
     b.n_total = a->n;
-    b.steps_per_fetch = p.steps_per_fetch;
+    b.steps_per_fetch = o->steps_per_fetch;
     b.queue = queue;
     e = (o->precision == MP_PREC_FP64) ? launch_track_fp64(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, block, 0, s)
                                        : launch_track_mixed(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, block, 0, s);

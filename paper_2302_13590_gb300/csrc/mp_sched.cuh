@@ -318,6 +318,8 @@ __device__ __forceinline__ bool path_start(const E& e, const S& s)
     return p.pathline && !p.cont && s.st != ST_SKIP && s.c >= 0;
 }
 
+constexpr int AXES_PARTICLES = 10;   // of a warp whose particles have three lanes each (lanes 30 and 31 none)
+
 template <class E, bool TS, bool PL>
 __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_static(E e)
 {
@@ -382,7 +384,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt_mask = (1u << lane) - 1u;
     const unsigned long long n = (unsigned long long)e.b.n_total;
-    const int S = e.b.steps_per_fetch > 0 ? e.b.steps_per_fetch : 1;
+    const int S = e.b.steps_per_fetch;
     long long q = -1;
     bool live = false;
     bool drained = false;
@@ -443,7 +445,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
 static_assert(sizeof(PathQ) % 16 == 0, "queue sizes are whole 16-byte words");
 
 template <class E, bool TS, bool PL>
-cudaError_t launch_variant(const E& e, int schedule, int block, int blocks_per_sm_cap, size_t smem, cudaStream_t st)
+cudaError_t launch_variant(E e, int schedule, int block, int blocks_per_sm_cap, size_t smem, cudaStream_t st)
 {
     auto kern = schedule == MP_SCHED_STATIC ? k_track_static<E, TS, PL> : k_track_dynamic<E, TS, PL>;
     cudaError_t err = cudaSuccess;
@@ -461,6 +463,14 @@ cudaError_t launch_variant(const E& e, int schedule, int block, int blocks_per_s
         if (per_sm < 1) per_sm = 1;
         if (blocks_per_sm_cap > 0 && per_sm > blocks_per_sm_cap) per_sm = blocks_per_sm_cap;
         if (grid > (long long)sms * per_sm) grid = (long long)sms * per_sm;
+        // Steps per fetch when the caller names none.  Bound by issue, a
+        // fetch costs what it holds the warp for: 16 steps while a lane tracks
+        // several particles in turn (mixed precision, 1e6 particles 5.70 ->
+        // 5.52 ms, 2e6 on 400x400x40 cells 21.3 -> 21.1 ms).  Bound by the
+        // FP64 pipe, an idle lane costs as much as a live one: 4 (1e6
+        // particles 23.19 ms, 23.41 with 16).  And 4 where most lanes have one
+        // particle (1e5 on a quadtree 0.96 ms, 1.19 with 16).
+        if (e.b.steps_per_fetch <= 0) e.b.steps_per_fetch = e.b.n_total >= 4 * grid * block ? E::FETCH : 4;
     }
     kern<<<(unsigned)grid, block, smem, st>>>(e);
     return cudaGetLastError();

@@ -147,6 +147,7 @@ template <bool ONE_REQ>
 struct UsgEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
+    static constexpr int FETCH = 4;            // steps per fetch
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevUsg u;
     Batch b;
