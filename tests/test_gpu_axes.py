@@ -1,7 +1,7 @@
-"""FP64 launches of few particles (three lanes each) and of many (one lane
-each) give every particle the same result, bit for bit: the same particles
-alone and repeated beyond the limit, over every option, at sizes around a
-warp's ten particles, in batches too."""
+"""Launches of few particles (three lanes each) and of many (one lane each)
+give every particle the same result, bit for bit, in FP64 and in mixed
+precision: the same particles alone and repeated beyond the limit, over every
+option, at sizes around a warp's ten particles, in batches too."""
 import numpy as np
 import pytest
 
@@ -10,7 +10,8 @@ from paper_2302_13590_gb300 import mp
 
 pytestmark = pytest.mark.gpu
 
-LIMIT = 18240   # particles of a launch up to which each has three lanes
+# particles of a launch up to which each has three lanes
+LIMIT = {mp.PREC_FP64: 18240, mp.PREC_MIXED: 30400}
 
 
 @pytest.fixture(scope="module")
@@ -46,10 +47,11 @@ def _run(ctx, fh, cells, frac, t0, times, kw):
     return ep, ts, pl, st
 
 
+@pytest.mark.parametrize("precision", [mp.PREC_FP64, mp.PREC_MIXED])
 @pytest.mark.parametrize("name", ["wells", "flat"])
 @pytest.mark.parametrize("n", [1, 9, 10, 11, 257])
 @pytest.mark.parametrize("option", ["endpoint", "times", "paths", "all", "weak sinks", "stop and resume", "step cap"])
-def test_few_equal_many(ctx, fields, name, n, option):
+def test_few_equal_many(ctx, fields, precision, name, n, option):
     f = fields[name]
     fh = ctx.field(f)
     rng = np.random.default_rng(n)
@@ -58,7 +60,7 @@ def test_few_equal_many(ctx, fields, name, n, option):
     ta = I.t_adv_of(f, 1e-4, 0.3)
     t0 = rng.random(n) * 0.2 * ta if option in ("all", "times") else None
     times = I.log_times(ta, 13) if option in ("times", "all", "weak sinks", "step cap") else None
-    kw = {"mode": mp.MODE_ENDPOINT | (mp.MODE_TIMESERIES if times is not None else 0)}
+    kw = {"mode": mp.MODE_ENDPOINT | (mp.MODE_TIMESERIES if times is not None else 0), "precision": precision}
     if option in ("paths", "all"):
         kw.update(mode=kw["mode"] | mp.MODE_PATHLINE, path_capacity=3000000)
     if option == "weak sinks":
@@ -68,9 +70,9 @@ def test_few_equal_many(ctx, fields, name, n, option):
     if option == "step cap":
         kw.update(max_steps=7)
     few = _run(ctx, fh, cells, frac, t0, times, kw)
-    rep = LIMIT // n + 1
+    rep = LIMIT[precision] // n + 1
     many = _run(ctx, fh, np.tile(cells, rep), np.tile(frac, (rep, 1)), None if t0 is None else np.tile(t0, rep), times, kw)
-    assert many[0]["t"].size > LIMIT >= n
+    assert many[0]["t"].size > LIMIT[precision] >= n
     for k, v in few[0].items():
         w = many[0][k].reshape(rep, n)
         assert (w.view(np.uint8) == np.ascontiguousarray(v).view(np.uint8).reshape(-1)).all(), k
@@ -87,18 +89,19 @@ def test_few_equal_many(ctx, fields, name, n, option):
     mp.mp_field_free(fh)
 
 
-def test_batch_of_few_equals_alone_among_many(ctx, fields):
+@pytest.mark.parametrize("precision", [mp.PREC_FP64, mp.PREC_MIXED])
+def test_batch_of_few_equals_alone_among_many(ctx, fields, precision):
     f = fields["wells"]
     fh = ctx.field(f)
     times = I.log_times(I.t_adv_of(f, 1e-4, 0.3), 9)
-    opts = [mp.make_opts(mode=mp.MODE_ENDPOINT | (mp.MODE_TIMESERIES if i % 2 else 0), times=times if i % 2 else None)
-            for i in range(12)]
+    opts = [mp.make_opts(mode=mp.MODE_ENDPOINT | (mp.MODE_TIMESERIES if i % 2 else 0), times=times if i % 2 else None,
+                         precision=precision) for i in range(12)]
     parts = [I.explicit_particles(f, 7 + 11 * i, seed=90 + i) for i in range(12)]
 
     def batch(extra):
         groups = [ctx.release_explicit(fh, c, x) for c, x in parts]
         more = [ctx.release_explicit(fh, *I.explicit_particles(f, extra, seed=3))] if extra else []
-        ids = mp.mp_track_batch(ctx.h, groups + more, opts + [mp.make_opts()] * len(more))
+        ids = mp.mp_track_batch(ctx.h, groups + more, opts + [mp.make_opts(precision=precision)] * len(more))
         out = []
         for i, (r, (c, _)) in enumerate(zip(ids, parts)):
             out.append(mp.mp_get_endpoints(ctx.h, r, c.size))
@@ -110,7 +113,7 @@ def test_batch_of_few_equals_alone_among_many(ctx, fields):
             mp.mp_group_free(g)
         return out
 
-    for a, b in zip(batch(0), batch(LIMIT + 1)):
+    for a, b in zip(batch(0), batch(LIMIT[precision] + 1)):
         for k in a:
             assert np.array_equal(np.ascontiguousarray(a[k]).view(np.uint8), np.ascontiguousarray(b[k]).view(np.uint8)), k
     mp.mp_field_free(fh)
