@@ -91,7 +91,7 @@ extern "C" {
 #define MP_SCHED_DYNAMIC 1      /* persistent warps refilled from a queue     */
 #define MP_SCHED_AUTO 2         /* the context's tuned launch (mp_autotune)
                                    for this field, precision and mode, else
-                                   dynamic, 128 threads                      */
+                                   dynamic, block and fetch chosen at launch */
 
 #define MP_TRACK_UPDATE_GROUP 1u /* write final state back into the group     */
 #define MP_TRACK_PASS_WEAK_SINKS 2u /* enter sink cells and leave them through

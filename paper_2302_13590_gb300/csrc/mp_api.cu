@@ -975,13 +975,12 @@ int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, const
         if (e == cudaSuccess) e = launch_zero_counters(b, s);
     }
     for (int i = 0; i < n && e == cudaSuccess && (ev & 1u); ++i) e = cudaEventRecord(rs[i]->k0, s);
-    const int blk = block > 0 ? block : 128;
     if (e == cudaSuccess) {
         const mp::DevField& fd = *mp::field_device_view(f);
-        if (f->usg) e = launch_track_usg(f->u, b, modes, schedule, blk, 0, s);
-        else e = (precision == MP_PREC_FP64)    ? launch_track_fp64(fd, b, modes, schedule, blk, 0, s)
-                 : (precision == MP_PREC_MIXED) ? launch_track_mixed(fd, b, modes, schedule, blk, 0, s)
-                                                : launch_track_mixed_f64t(fd, b, modes, schedule, blk, 0, s);
+        if (f->usg) e = launch_track_usg(f->u, b, modes, schedule, block, s);
+        else e = (precision == MP_PREC_FP64)    ? launch_track_fp64(fd, b, modes, schedule, block, s)
+                 : (precision == MP_PREC_MIXED) ? launch_track_mixed(fd, b, modes, schedule, block, s)
+                                                : launch_track_mixed_f64t(fd, b, modes, schedule, block, s);
         if (e == cudaSuccess) e = mp::launch_spread_window(b, s);
     }
     for (int i = 0; i < n && e == cudaSuccess && (ev & 2u); ++i) e = cudaEventRecord(rs[i]->k1, s);
@@ -1000,7 +999,7 @@ void resolve_launch(mp_ctx* ctx, const mp_field* f, int precision, bool ts, cons
     *spf = o.steps_per_fetch;
     if (*sched != MP_SCHED_AUTO) return;
     *sched = MP_SCHED_DYNAMIC;
-    *blk = 128;
+    *blk = 0;
     *spf = 0;
     std::lock_guard<std::mutex> lk(ctx->mu);
     auto it = ctx->tuned.find(TuneKey{f, precision, ts ? 1 : 0});
@@ -1766,8 +1765,8 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
         int sched = 0, blk = 0, spf = 0;
         resolve_launch(ctx, f, prec, (modes[p] & mp::MODE_TS) != 0, opts[sel[p][0]], &sched, &blk, &spf);
         bat[p].steps_per_fetch = spf;
-        e = prec == MP_PREC_FP64 ? mp::launch_track_fp64(fd, bat[p], modes[p], sched, blk > 0 ? blk : 128, 0, cs)
-                                 : mp::launch_track_mixed(fd, bat[p], modes[p], sched, blk > 0 ? blk : 128, 0, cs);
+        e = prec == MP_PREC_FP64 ? mp::launch_track_fp64(fd, bat[p], modes[p], sched, blk, cs)
+                                 : mp::launch_track_mixed(fd, bat[p], modes[p], sched, blk, cs);
         if (e == cudaSuccess) e = mp::launch_spread_window(bat[p], cs);
     }
     cudaGraph_t graph = nullptr;

@@ -444,6 +444,7 @@ template <bool ONE_REQ>
 struct F64Engine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
+    static constexpr bool EVEN_ROUNDS = true;   // more particles than lanes: rounds of even size
     static constexpr int FETCH = 4;            // steps per fetch
     // blocks of 256 threads to keep resident per SM (0: no target; the
     // kernels are FP64-pipe bound)
@@ -1192,17 +1193,16 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                              int blocks_per_sm_cap, cudaStream_t s)
+cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_total <= 0) return cudaSuccess;
     const bool few = b.n_total <= AXES_MAX;
     if (b.n_reqs == 1) {
         const F64Engine<true> e{f, b};
-        return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+        return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, s);
     }
     const F64Engine<false> e{f, b};
-    return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, s);
 }
 
 }  // namespace mp

@@ -277,8 +277,7 @@ cudaError_t launch_build_usg(const DevUsg& u, UsgCell* cell, UsgGeo* geo, double
                              const double* box, const double* por, cudaStream_t s);
 cudaError_t launch_release_explicit_usg(const DevUsg& u, const DevState& st, long long n, const int32_t* cell,
                                         const double* local, const double* t0, cudaStream_t s);
-cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block,
-                             int blocks_per_sm_cap, cudaStream_t s);
+cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
 
 // one group's box release, as a device descriptor (graph replays read it)
 struct BoxRelease {
@@ -299,16 +298,13 @@ cudaError_t launch_release_box(const DevField& f, const DevState& st, long long 
 cudaError_t launch_release_explicit(const DevField& f, const DevState& st, long long n, const int32_t* cell,
                                     const double* local, const double* t0, cudaStream_t s);
 // ts: true if any request of the batch writes timeseries records
-cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                              int blocks_per_sm_cap, cudaStream_t s);
-cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                               int blocks_per_sm_cap, cudaStream_t s);
+cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
+cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
 // zero the counters of a batch's requests (n_reqs > 1)
 cudaError_t launch_zero_counters(const Batch& b, cudaStream_t s);
 // copy the first request's launch window into the other requests of a batch
 cudaError_t launch_spread_window(const Batch& b, cudaStream_t s);
-cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                               int blocks_per_sm_cap, cudaStream_t s);
+cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
 
 // device-to-device copies of a request's arrays into the caller's, as one launch
 struct CopyItem {

@@ -11,17 +11,16 @@ namespace mp {
 // 328 / 294; the FP64 form's line is lower, its warps wait for one FP64 unit).
 constexpr long long MIXED_AXES_MAX = 20 * 152 * AXES_PARTICLES;
 
-cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                               int blocks_per_sm_cap, cudaStream_t s)
+cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_total <= 0) return cudaSuccess;
     const bool few = b.n_total <= MIXED_AXES_MAX;
     if (b.n_reqs == 1) {
         const MixEngine<false, true> e{f, b};
-        return few ? launch_axes_mixed(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+        return few ? launch_axes_mixed(e, modes, s) : launch_tracking(e, modes, schedule, block, s);
     }
     const MixEngine<false, false> e{f, b};
-    return few ? launch_axes_mixed(e, modes, s) : launch_tracking(e, modes, schedule, block, blocks_per_sm_cap, s);
+    return few ? launch_axes_mixed(e, modes, s) : launch_tracking(e, modes, schedule, block, s);
 }
 
 }  // namespace mp

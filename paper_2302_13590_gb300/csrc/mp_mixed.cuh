@@ -45,6 +45,7 @@ template <bool F64T, bool ONE_REQ>
 struct MixEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = true;   // records wait in the lane's own slots
+    static constexpr bool EVEN_ROUNDS = false;   // (issue bound: as many warps as fit)
     static constexpr int FETCH = 16;          // steps per fetch while a lane tracks several particles in turn
     // What bounds it: issue (70 % of the slots; ALU instructions take two
     // cycles each), with 32 warps an SM hiding the rest, so four blocks of 256

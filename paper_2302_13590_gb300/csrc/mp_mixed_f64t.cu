@@ -6,12 +6,11 @@
 
 namespace mp {
 
-cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block,
-                                    int blocks_per_sm_cap, cudaStream_t s)
+cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_reqs == 1)
-        return launch_tracking(MixEngine<true, true>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
-    return launch_tracking(MixEngine<true, false>{f, b}, modes, schedule, block, blocks_per_sm_cap, s);
+        return launch_tracking(MixEngine<true, true>{f, b}, modes, schedule, block, s);
+    return launch_tracking(MixEngine<true, false>{f, b}, modes, schedule, block, s);
 }
 
 }  // namespace mp

@@ -134,7 +134,6 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     p.cont = 0;
     p.last = 1;
     split_ff(p.t_stop, p.tstop_hi, p.tstop_lo);
-    const int block = o->block > 0 ? o->block : 128;
     const DevField& fd = *mp::field_device_view(f);
     Batch b{};
     b.one.in = st;
@@ -144,8 +143,8 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     b.n_total = a->n;
     b.steps_per_fetch = o->steps_per_fetch;
     b.queue = queue;
-    e = (o->precision == MP_PREC_FP64) ? launch_track_fp64(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, block, 0, s)
-                                       : launch_track_mixed(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, block, 0, s);
+    e = (o->precision == MP_PREC_FP64) ? launch_track_fp64(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, o->block, s)
+                                       : launch_track_mixed(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, o->block, s);
     if (e != cudaSuccess) return na_fail(MP_ERR_CUDA, std::string("mp_track_noalloc: launch: ") + cudaGetErrorString(e));
     if (stats) {
         unsigned long long h[N_COUNTERS];

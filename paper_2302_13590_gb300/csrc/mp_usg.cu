@@ -147,6 +147,7 @@ template <bool ONE_REQ>
 struct UsgEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
+    static constexpr bool EVEN_ROUNDS = true;   // more particles than lanes: rounds of even size
     static constexpr int FETCH = 4;            // steps per fetch
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevUsg u;
@@ -622,11 +623,10 @@ struct UsgEngine {
     }
 };
 
-cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block,
-                             int blocks_per_sm_cap, cudaStream_t s)
+cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
-    if (b.n_reqs == 1) return launch_tracking(UsgEngine<true>{u, b}, modes, schedule, block, blocks_per_sm_cap, s);
-    return launch_tracking(UsgEngine<false>{u, b}, modes, schedule, block, blocks_per_sm_cap, s);
+    if (b.n_reqs == 1) return launch_tracking(UsgEngine<true>{u, b}, modes, schedule, block, s);
+    return launch_tracking(UsgEngine<false>{u, b}, modes, schedule, block, s);
 }
 
 }  // namespace mp
