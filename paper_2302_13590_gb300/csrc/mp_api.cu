@@ -340,6 +340,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     const size_t o_delc = off; off = align256(off + sizeof(double) * nr);
     const size_t o_dz = off; off = align256(off + sizeof(double) * nl);
     const size_t o_ax = off; off = align256(off + sizeof(AxisCell) * (nc + nr + nl));
+    const size_t o_inv = off; off = align256(off + sizeof(double) * (nc + nr + nl));
     const size_t o_xf = off; off = align256(off + sizeof(double) * (nc + 1));
     const size_t o_yf = off; off = align256(off + sizeof(double) * (nr + 1));
     const size_t o_zf = off; off = align256(off + sizeof(double) * (nl + 1));
@@ -380,12 +381,14 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     memcpy(host(o_delc), d->delc, sizeof(double) * nr);
     memcpy(host(o_dz), d->dz, sizeof(double) * nl);
     AxisCell* axc = reinterpret_cast<AxisCell*>(host(o_ax));
+    double* inv = host(o_inv);
     int no_screen = 0;
     auto add_axis = [&](const double* D, long long m, double org, double* face) {
         face[0] = org;
         for (long long a = 0; a < m; ++a) {
             face[a + 1] = face[a] + D[a];
             *axc++ = AxisCell{D[a], host_f32_trunc(D[a]), 0.0f};
+            *inv++ = 1.0 / D[a];
             if (D[a] > SCREEN_MAX_D) no_screen = 1;
         }
     };
@@ -421,6 +424,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     v.delc = reinterpret_cast<double*>(buf + o_delc);
     v.dz = reinterpret_cast<double*>(buf + o_dz);
     v.ax = reinterpret_cast<AxisCell*>(buf + o_ax);
+    v.inv = reinterpret_cast<double*>(buf + o_inv);
     v.no_screen = no_screen;
     v.xf = reinterpret_cast<double*>(buf + o_xf);
     v.yf = reinterpret_cast<double*>(buf + o_yf);

@@ -593,4 +593,57 @@ __device__ __forceinline__ int screen(float e0, float e1, float e2, unsigned rea
     return a0;
 }
 
+// ---------------------------------------------------------------------------
+// quotients and conversions of the field records (once per cell; the same
+// values as the IEEE operations, on fewer FP64 instructions)
+// ---------------------------------------------------------------------------
+
+// |D| in [2^-60, 2^60): divisors that the forms below take
+__device__ __forceinline__ bool plain_divisor(double D)
+{
+    unsigned lo, hi;
+    words(D, lo, hi);
+    return hi_abs(hi) - 0x3c300000u < 0x07800000u;
+}
+
+// a / D from y = RN(1 / D), D a plain divisor: two corrections by the exact
+// remainder, the first to within an ulp, the second to the rounded quotient
+// (Markstein, as above); five instructions where the division takes about
+// nine.  Magnitudes near the ends of the range take the division.
+__device__ __forceinline__ double div_by(double a, double D, double y)
+{
+    unsigned lo, hi;
+    words(a, lo, hi);
+    if (zero_w(lo, hi)) return a;
+    if (hi_abs(hi) - 0x0c700000u >= 0x67100000u) return a / D;   // 2^-824 <= |a| < 2^825
+    const double q0 = a * y;
+    const double q1 = fma(fma(-D, q0, a), y, q0);
+    return fma(fma(-D, q1, a), y, q1);
+}
+
+// (float)x rounded to nearest even, on the ALU where the result is normal
+__device__ __forceinline__ float f32_rn(double x)
+{
+    unsigned lo, hi;
+    words(x, lo, hi);
+    if (zero_w(lo, hi)) return __uint_as_float(hi);
+    if (hi_abs(hi) - 0x38100000u >= 0x0fd00000u) return (float)x;   // 2^-126 <= |x| < 2^127
+    const unsigned fb = __float_as_uint(trunc_normal(lo, hi)), rem = lo & 0x1fffffffu;
+    return __uint_as_float(fb + ((rem > 0x10000000u || (rem == 0x10000000u && (fb & 1u))) ? 1u : 0u));
+}
+
+// (float)(v / D) from y = RN(1 / D), D a plain divisor: v y is within two ulp
+// of the quotient, which decides the FP32 value unless it lies that close to
+// the middle between two
+__device__ __forceinline__ float quot_f32(double v, double D, double y)
+{
+    unsigned lo, hi;
+    words(v, lo, hi);
+    if (zero_w(lo, hi)) return __uint_as_float(hi);
+    words(v * y, lo, hi);
+    const unsigned rem = lo & 0x1fffffffu;
+    if (hi_abs(hi) - 0x38100000u >= 0x0fd00000u || rem - 0x0ffffffcu < 9u) return (float)(v / D);
+    return __uint_as_float(__float_as_uint(trunc_normal(lo, hi)) + (rem >> 28));
+}
+
 }  // namespace mp

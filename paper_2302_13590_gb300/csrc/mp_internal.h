@@ -76,6 +76,7 @@ struct DevField {
     const double* delc;
     const double* dz;
     const AxisCell* ax;   // sizes of the columns, then the rows, then the layers
+    const double* inv;    // their reciprocals
     const double* xf;  // [ncol+1]
     const double* yf;  // [nrow+1]
     const double* zf;  // [nlay+1]

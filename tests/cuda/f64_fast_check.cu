@@ -2,7 +2,9 @@
 // ones, bit for bit: fast_log1p against series_log1p (around every row edge,
 // sqrt2 and the ends of the table too), f64_move_fast against f64_move, the
 // word forms of the FP32 truncation against f32_trunc, the FP32 reciprocal
-// against __frcp_rn on every significand, the time keys against the FP64 order, and the screened exit axis against all three exact times.
+// against __frcp_rn on every significand, the time keys against the FP64
+// order, the screened exit axis against all three exact times, the quotients
+// and conversions of the field records against the IEEE ones.
 // Prints the mismatch counts and exits non-zero on any.
 #include <cstdio>
 
@@ -86,6 +88,19 @@ __global__ void check(unsigned long long* bad, unsigned long long n)
         const float rx = __uint_as_float((unsigned)(i & 0x7fffffu) | ((7u + (unsigned)(mix64(i >> 23) % 240)) << 23) |
                                          ((unsigned)(r >> 40) << 31));
         if (__float_as_uint(rcp_rn_normal(rx)) != __float_as_uint(__frcp_rn(rx))) atomicAdd(bad + 6, 1ULL);
+        // the field records' quotients and conversions against IEEE ones
+        {
+            const double Dd = spread(mix64(r + 40), -62, 62), yd = 1.0 / Dd;
+            double v = (c & 32 ? -1.0 : 1.0) * (c % 3 ? spread(mix64(r + 41), -40, 10) : spread(mix64(r + 41), -1074, 1023));
+            if (c % 5 == 0) v = Dd * (double)__uint_as_float((unsigned)(r >> 20) & 0x3fffffffu);           // near FP32 values
+            if (c % 5 == 1) v = Dd * ((double)__uint_as_float(((unsigned)(r >> 20) & 0x3fffffffu) | 0x20000000u) * (1.0 + 0x1p-24));   // and middles
+            if (c % 43 == 0) v = c & 64 ? 0.0 : -0.0;
+            if (plain_divisor(Dd)) {
+                if (!same(div_by(v, Dd, yd), v / Dd)) atomicAdd(bad + 7, 1ULL);
+                if (__float_as_uint(quot_f32(v, Dd, yd)) != __float_as_uint((float)(v / Dd))) atomicAdd(bad + 7, 1ULL);
+            }
+            if (__float_as_uint(f32_rn(v)) != __float_as_uint((float)v)) atomicAdd(bad + 7, 1ULL);
+        }
         // keys of times
         const double a = (c & 8 ? 1.0 : -1.0) * spread(mix64(r + 7), -3, 3) * (c % 23 == 0 ? 0.0 : 1.0) + 0.0;
         const double b = c % 29 == 0 ? a : (c & 16 ? 1.0 : -1.0) * spread(mix64(r + 8), -3, 3) * (c % 31 == 0 ? 0.0 : 1.0);
@@ -151,8 +166,8 @@ int main()
     unsigned long long h[8] = {0};
     cudaMemcpy(h, bad, sizeof h, cudaMemcpyDeviceToHost);
     const cudaError_t e = cudaDeviceSynchronize();
-    printf("%s log1p %llu move %llu trunc %llu keys %llu face %llu screen %llu rcp %llu\n", cudaGetErrorString(e),
-           h[0], h[1], h[2], h[3], h[4], h[5], h[6]);
+    printf("%s log1p %llu move %llu trunc %llu keys %llu face %llu screen %llu rcp %llu quotients %llu\n",
+           cudaGetErrorString(e), h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7]);
     cudaFree(bad);
-    return (e == cudaSuccess && !(h[0] | h[1] | h[2] | h[3] | h[4] | h[5] | h[6])) ? 0 : 1;
+    return (e == cudaSuccess && !(h[0] | h[1] | h[2] | h[3] | h[4] | h[5] | h[6] | h[7])) ? 0 : 1;
 }
