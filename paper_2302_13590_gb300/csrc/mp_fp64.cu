@@ -455,7 +455,7 @@ struct F64Engine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
     static constexpr bool EVEN_ROUNDS = true;   // more particles than lanes: rounds of even size
-    static constexpr int FETCH = 4;            // steps per fetch
+    static constexpr int FETCH = 8;            // steps per fetch
     // blocks of 256 threads to keep resident per SM (0: no target; the
     // kernels are FP64-pipe bound)
     static constexpr int min_blocks(bool, bool, bool) { return 0; }

@@ -46,7 +46,7 @@ struct MixEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = true;   // records wait in the lane's own slots
     static constexpr bool EVEN_ROUNDS = false;   // (issue bound: as many warps as fit)
-    static constexpr int FETCH = 16;          // steps per fetch while a lane tracks several particles in turn
+    static constexpr int FETCH = 16;          // steps per fetch
     // What bounds it: issue (70 % of the slots; ALU instructions take two
     // cycles each), with 32 warps an SM hiding the rest, so four blocks of 256
     // threads at 64 registers and nothing spilled.  For that the state is kept

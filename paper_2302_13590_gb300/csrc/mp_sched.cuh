@@ -11,6 +11,13 @@
 //             This is the GPU form of OpenMP `dynamic` (a new particle is
 //             taken on completion of the current one) and keeps warps full
 //             through the heavy tail of slow particles.
+// A particle that ended is written out where its warp fetches (static: after
+// the warp's last step), together with the others that ended since then: its
+// lane waits for that anyway, and writing each out in the step in which it
+// ends held the 31 other lanes for its endpoint, once for every particle
+// instead of once for a fetch.  Static 5.24 -> 5.02 ms, dynamic 5.49 -> 5.27
+// (1e6 particles, 200x200x20 cells, mixed precision), FP64 23.19 -> 22.95,
+// quadtree of 1e6 7.40 -> 6.84, 240,000 of a batch 1.18 -> 1.15.
 // Per-status counts and cell-step totals (the paper's `reduction` counters,
 // Fig. 2) go to shared-memory atomics and one global atomic per block.
 #pragma once
@@ -340,28 +347,23 @@ __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_sta
     s.steps = 0;
     s.st = ST_SKIP;
     s.c = -1;
-    bool live = false, ended = false, loaded = false;
+    bool live = false, mine = false, loaded = false;   // mine: the lane has an endpoint to write
     if (g < e.b.n_total) {
         const int r = request_of(e, g, q);
         e.template load<TS>(r, q, s);
         live = s.st == MP_ST_ACTIVE;
-        ended = !live && s.st != ST_SKIP;
+        mine = s.st != ST_SKIP;
         loaded = true;
     }
     if (PL) pl_push(e, P, pcount, s, q, loaded && path_start(e, s), s.st == MP_ST_TIME ? MP_ST_ACTIVE : s.st);
-    if (TS) tail_fill(e, s, q, ended && !paused(e, s));
-    if (ended) e.template finish<TS>(q, s, s_cnt);
     while (__any_sync(FULL, live)) {
         const unsigned before = s.steps;
         e.template step<TS>(q, s, live, Q, qcount);
         if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.req(s.r).p.pathline, s.st);
-        ended = live && s.st != MP_ST_ACTIVE;
-        if (TS) tail_fill(e, s, q, ended && !paused(e, s));
-        if (ended) {
-            e.template finish<TS>(q, s, s_cnt);
-            live = false;
-        }
+        live = live && s.st == MP_ST_ACTIVE;
     }
+    if (TS) tail_fill(e, s, q, mine && !paused(e, s));
+    if (mine) e.template finish<TS>(q, s, s_cnt);
     if (TS) rec_finish(e, Q, qcount);
     if (PL) pl_flush(e, P, pcount);
     flush_counters(e, s_cnt);
@@ -386,8 +388,7 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     const unsigned long long n = (unsigned long long)e.b.n_total;
     const int S = e.b.steps_per_fetch;
     long long q = -1;
-    bool live = false;
-    bool drained = false;
+    bool live = false, mine = false, drained = false;   // mine: the lane holds a particle that is not finished yet
     typename E::State s;
     s.r = 0;
     s.steps = 0;
@@ -395,41 +396,40 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     s.c = -1;
     while (true) {
         const unsigned idle = __ballot_sync(FULL, !live);
-        bool ended = false, loaded = false;
-        if (idle && !drained) {
-            const unsigned cnt = __popc(idle);
-            unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(e.b.queue, (unsigned long long)cnt);
-            base = __shfl_sync(FULL, base, 0);
-            if (base + cnt >= n) drained = true;
-            if (!live) {
-                const unsigned long long qq = base + __popc(idle & lt_mask);
-                if (qq < n) {
-                    const int r = request_of(e, (long long)qq, q);
-                    e.template load<TS>(r, q, s);
-                    live = s.st == MP_ST_ACTIVE;
-                    ended = !live && s.st != ST_SKIP;
-                    loaded = true;
+        if (idle) {
+            const bool ended = mine && !live;
+            if (TS) tail_fill(e, s, q, ended && !paused(e, s));
+            if (ended) e.template finish<TS>(q, s, s_cnt);
+            mine = live;
+            if (drained) {
+                if (idle == FULL) break;
+            } else {
+                const unsigned cnt = __popc(idle);
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(e.b.queue, (unsigned long long)cnt);
+                base = __shfl_sync(FULL, base, 0);
+                if (base + cnt >= n) drained = true;
+                bool loaded = false;
+                if (!live) {
+                    const unsigned long long qq = base + __popc(idle & lt_mask);
+                    if (qq < n) {
+                        const int r = request_of(e, (long long)qq, q);
+                        e.template load<TS>(r, q, s);
+                        live = s.st == MP_ST_ACTIVE;
+                        mine = s.st != ST_SKIP;
+                        loaded = true;
+                    }
                 }
+                if (PL)
+                    pl_push(e, P, pcount, s, q, loaded && path_start(e, s), s.st == MP_ST_TIME ? MP_ST_ACTIVE : s.st);
+                if (!__any_sync(FULL, live)) continue;
             }
-        }
-        if (PL) pl_push(e, P, pcount, s, q, loaded && path_start(e, s), s.st == MP_ST_TIME ? MP_ST_ACTIVE : s.st);
-        if (TS) tail_fill(e, s, q, ended && !paused(e, s));
-        if (ended) e.template finish<TS>(q, s, s_cnt);
-        if (!__any_sync(FULL, live)) {
-            if (drained) break;
-            continue;
         }
         for (int it = 0; it < S; ++it) {
             const unsigned before = s.steps;
             e.template step<TS>(q, s, live, Q, qcount);
             if (PL) pl_push(e, P, pcount, s, q, live && s.steps != before && e.req(s.r).p.pathline, s.st);
-            ended = live && s.st != MP_ST_ACTIVE;
-            if (TS) tail_fill(e, s, q, ended && !paused(e, s));
-            if (ended) {
-                e.template finish<TS>(q, s, s_cnt);
-                live = false;
-            }
+            live = live && s.st == MP_ST_ACTIVE;
         }
     }
     if (TS) rec_finish(e, Q, qcount);
@@ -480,14 +480,15 @@ cudaError_t launch_variant(E e, int schedule, int block, size_t smem, cudaStream
             }
         }
         if (grid > (long long)sms * per_sm) grid = (long long)sms * per_sm;
-        // Steps per fetch when the caller names none.  Bound by issue, a
-        // fetch costs what it holds the warp for: 16 steps while a lane tracks
-        // several particles in turn (mixed precision, 1e6 particles 5.70 ->
-        // 5.52 ms, 2e6 on 400x400x40 cells 21.3 -> 21.1 ms).  Bound by the
-        // FP64 pipe, an idle lane costs as much as a live one: 4 (1e6
-        // particles 23.19 ms, 23.41 with 16).  And 4 where most lanes have one
-        // particle (1e5 on a quadtree 0.96 ms, 1.19 with 16).
-        if (e.b.steps_per_fetch <= 0) e.b.steps_per_fetch = e.b.n_total >= 4 * grid * block ? E::FETCH : 4;
+        // Steps per fetch when the caller names none: a fetch holds the warp
+        // for the loads, and the ends, of a few of its lanes; between two of
+        // them a lane whose particle ended waits.  Bound by issue (mixed
+        // precision) 16 is best (1e6 particles 278 steps the mean path, 4: 5.55,
+        // 8: 5.39, 16: 5.27 ms; 46 steps the mean path 0.62, 0.58, 0.57; 240,000
+        // of a batch 1.15, 1.11, 1.08), bound by the FP64 pipe, where an idle
+        // lane costs as much as a live one, 8 (1e6 on a quadtree, 54 steps the
+        // mean path 6.84, 6.65, 6.72 ms; 1e6 of 278 steps 22.95, 22.93, 23.06).
+        if (e.b.steps_per_fetch <= 0) e.b.steps_per_fetch = E::FETCH;
     }
     kern<<<(unsigned)grid, block, smem, st>>>(e);
     return cudaGetLastError();

@@ -148,7 +148,7 @@ struct UsgEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = false;   // records go through the warp's queue
     static constexpr bool EVEN_ROUNDS = true;   // more particles than lanes: rounds of even size
-    static constexpr int FETCH = 4;            // steps per fetch
+    static constexpr int FETCH = 8;            // steps per fetch
     static constexpr int min_blocks(bool, bool, bool) { return 0; }
     DevUsg u;
     Batch b;
