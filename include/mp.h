@@ -537,11 +537,13 @@ int mp_track_launches(const mp_track_opts* o, int32_t* launches);
  * mp_get_endpoints (ep: any pointer may be NULL) and, when o->mode has
  * MP_MODE_TIMESERIES and ts is not NULL, the [n_times][n] records into
  * ts (row stride n).  Particles move independently (Methods, "MODPATH"), so
- * the call splits them into n_chunks contiguous chunks (n_chunks <= 0:
- * chunks of about 128 K particles, 2 to 16 of them) and runs chunk c's
- * copy-in, release, tracking and copy-out in order on the second of two
- * internal streams when c is odd, the first otherwise: the result copies of
- * one chunk overlap the tracking of the next.  MP_SCHED_AUTO runs the chunks
+ * the call splits them into n_chunks contiguous chunks (n_chunks <= 0: one
+ * chunk up to 262144 particles in FP64, 131072 in the other precisions,
+ * else chunks of about 128 K particles, at most 16 of them).  Chunk c's
+ * copy-in, release and tracking run in order on the second of two internal
+ * streams when c is odd, the first otherwise, and its copy-out on a third:
+ * every chunk is launched before the first result is read, and the result
+ * copies of one chunk overlap the tracking of the next.  MP_SCHED_AUTO runs the chunks
  * with the static schedule (its blocks retire as their particles finish, so
  * the next chunk's blocks take their SMs).  The results are those of one
  * mp_release_group + mp_track + mp_get_endpoints / mp_get_timeseries over
@@ -551,7 +553,7 @@ int mp_track_launches(const mp_track_opts* o, int32_t* launches);
  * the caller; the call returns after the last copy has landed (bounded
  * wait, 60 s) and frees what it allocated.  stats (may be NULL): the sums of
  * the chunks' counters; kernel_ms = device time from the first chunk's
- * start to the last chunk's last copy.  The two streams belong to the
+ * start to the last chunk's last copy.  The streams belong to the
  * context and are kept for its later calls (the chunks' buffers are then
  * reused in stream order); calls on one context run one at a time.
  * MP_MODE_PATHLINE is rejected.

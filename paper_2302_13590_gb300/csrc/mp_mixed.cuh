@@ -55,9 +55,11 @@ struct MixEngine {
     // slots.  Measured on 1e6 particles, 200x200x20 cells, 50 output times:
     // persistent schedule 6.48 -> 5.70 ms (76 registers and the warp's queue
     // before; with that queue at 64 registers 5.82), static 5.48 -> 5.23 ms;
-    // 2e6 particles, 400x400x40 cells, 20 times 25.1 -> 21.3 ms.  A batch's
-    // kernels need 80 registers (the descriptors are read through a table):
-    // three blocks.
+    // 2e6 particles, 400x400x40 cells, 20 times 25.1 -> 21.3 ms.  (With the
+    // fetch of mp_sched.cuh: 5.26, 5.02 and 20.4 ms.)  A batch's persistent
+    // kernel keeps 80 registers (the descriptors are read through a table):
+    // three blocks; 240,000 particles of 24 requests 1.07 ms, at 64 registers
+    // and four blocks 1.14.
     static constexpr int min_blocks(bool dynamic, bool, bool pl) { return pl ? 0 : (dynamic ? (ONE ? 4 : 3) : 4); }
     DevField f;
     Batch b;

@@ -178,8 +178,8 @@ __device__ __forceinline__ void rq_push(const E& e, typename E::RecQ& Q, int& qc
 // a common queue in every step than on the records), and the warp evaluates
 // all of them when a lane has no room.  A list of the filled slots, built from
 // ballots, gives every lane one request at a time.  Three slots run as fast as
-// four (5.83 against 5.70 ms on the case above the mixed engine), two slower
-// (6.10), six as four, at more shared memory.
+// four (5.83 against 5.70 ms on the case above the mixed engine, when these
+// were compared), two slower (6.10), six as four, at more shared memory.
 constexpr int REC_SLOTS = 4;
 
 template <class E>
