@@ -1036,10 +1036,14 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
         double xn = f64_move_fast(c.A, c.iA, c.D, vp, x, tmin, again);
         again = again && a != ax;
         // an event: an output time or the stop time in the step, no exit, a
-        // path that ends here, the step cap, a motion for the general form
+        // path that ends here, the step cap, a motion for the general form, a
+        // candidate whose exact time is not finite: if that is the leading
+        // one, the others' times are not bounded by it, so every reachable
+        // axis decides, as in the one-lane engine
+        const bool open = use && !has && !exact && em >= 0.0f;
         const bool ev = go && (ax < 0 || tkey(t_end) >= s.tev);
-        if (__any_sync(FULL, ev || (live && (!go || !enter || again)))) {
-            if (__any_sync(FULL, go && !exact && ax < 0 && face != 0)) {   // the leading time was not usable
+        if (__any_sync(FULL, open || ev || (live && (!go || !enter || again)))) {
+            if (__any_sync(FULL, open)) {
                 exact = true;
                 continue;
             }
