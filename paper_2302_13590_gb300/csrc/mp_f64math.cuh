@@ -470,6 +470,12 @@ __device__ __forceinline__ double f64_face_dist(int face, double D, double pp)
     return face > 0 ? D - pp : neg(pp);
 }
 
+// 0 <= pp <= D as unsigned words (a set sign is the largest; D > 0)
+__device__ __forceinline__ bool f64_inside(double pp, double D)
+{
+    return (unsigned long long)bits(pp) <= (unsigned long long)bits(D);
+}
+
 // particle velocity at offset pp from face 1: v1 + A pp, one rounding
 __device__ __forceinline__ double f64_vel(double v1, double A, double pp) { return fma(A, pp, v1); }
 

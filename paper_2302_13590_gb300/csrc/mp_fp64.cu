@@ -14,6 +14,7 @@
 // neighbour across it, until a stopping condition holds (Methods, "MODPATH").
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "mp_internal.h"
 #include "mp_sched.cuh"
@@ -478,7 +479,8 @@ struct F64Engine {
         double x0, x1, x2;   // offsets (m) from the cell's low faces
         double t;
         unsigned steps;
-        unsigned cap;     // the request's step cap (its low 32 bits' range; the full one decides)
+        unsigned cap;     // the request's step cap (its low 32 bits' range; the full one decides); 0: an
+                          // offset was handed in outside its cell, and every axis is evaluated exactly
         unsigned long long h;
         int kn;
         int st;
@@ -567,6 +569,11 @@ struct F64Engine {
         s.in_sink = 0;
         if (s.c >= 0 && (long long)s.c < f.ncell) {
             split_cell(f, s.c, s.k, s.i, s.j);
+            // a caller's own arrays (they come without step counts) may hold
+            // offsets outside the cell, rounded ones for instance
+            if (!in.steps && !(f64_inside(s.x0, __ldg(f.delr + s.j)) && f64_inside(s.x1, __ldg(f.delc + s.i)) &&
+                               f64_inside(s.x2, __ldg(f.dz + s.k))))
+                s.cap = 0u;
             s.h = (s.steps && in.hash) ? in.hash[q] : fnv_step(s.h, s.c);
             // a resumed particle may sit inside a sink cell it entered with
             // pass-through; a moving particle whose cell is not active under
@@ -667,7 +674,8 @@ struct F64Engine {
         int f0 = 0, f1 = 0, f2 = 0, ax = -1;
         unsigned nb = 0;
         if (live) {
-            if (s.steps >= s.cap && (long long)s.steps >= p.max_steps) {
+            const bool odd = s.steps >= s.cap;   // (off the fast path: at the cap, or its 0)
+            if (odd && (long long)s.steps >= p.max_steps) {
                 s.st = MP_ST_STEP_CAP;
             } else if ((unsigned)s.c >= (unsigned)f.ncell) {
                 atomicCAS(o.counters + COUNTER_ERR, 0ULL, (unsigned long long)q + 1ULL);
@@ -711,7 +719,7 @@ struct F64Engine {
                 const float t1 = f32_estimate(d1, trunc_normal(l1, h1), g1.y, f1 > 0 ? g1.x : g0.w);
                 const float t2 = f32_estimate(d2, trunc_normal(l2, h2), g2.x, f2 > 0 ? g1.w : g1.z);
                 const unsigned reach = (f0 ? 1u : 0u) | (f1 ? 2u : 0u) | (f2 ? 4u : 0u);
-                const bool doubt = f.no_screen || (f0 && !(vel_trusted(h0) && t0 < CUDART_INF_F)) ||
+                const bool doubt = f.no_screen || odd || (f0 && !(vel_trusted(h0) && t0 < CUDART_INF_F)) ||
                                    (f1 && !(vel_trusted(h1) && t1 < CUDART_INF_F)) ||
                                    (f2 && !(vel_trusted(h2) && t2 < CUDART_INF_F));
                 unsigned rest;
@@ -986,9 +994,12 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
     c.D = 1.0;
     if (live) c = read_axis(f, s.c, a, axis_at + ix);
     const int next1 = base + (a == 2 ? 0 : a + 1), next2 = base + (a == 0 ? 2 : a - 1);
-    bool exact = false;   // every reachable axis in this step
     bool going = __any_sync(FULL, live);
-    while (going) {
+    // One step of the warp's particles.  False: nothing was done, the step has
+    // to be made with every reachable axis's exact time (EXACT; rare, and a
+    // copy of its own so that the common step carries no test for it).
+    auto step = [&](auto every) -> bool {
+        constexpr bool EXACT = decltype(every)::value;
         const TrackParams& p = e.req(s.r).p;
         const bool go = live && !(s.steps >= s.cap && (long long)s.steps >= p.max_steps);
         // velocity, reachable face, FP32 estimate of the time to it (as in
@@ -1009,11 +1020,11 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
         const float em = fminf(est, fminf(__shfl_sync(FULL, est, next1), __shfl_sync(FULL, est, next2)));
         // the exact time of the axes within 2^-10 of the smallest estimate
         // (all reachable ones in doubt); the smallest wins, ties to the lower axis
-        const bool use = face != 0 && (exact || em < 0.0f || est <= em * (1.0f + 0.0009765625f));
+        const bool use = face != 0 && (EXACT || em < 0.0f || est <= em * (1.0f + 0.0009765625f));
         const double te = f64_exit_time_d(c.A, c.iA, d, face ? vp : 1.0, use);
         words(te, lo, hi);
-        const bool has = use && hi_abs(hi) < 0x7ff00000u;
-        const unsigned long long key = has ? (unsigned long long)hi_abs(hi) << 32 | lo : 0x7ff0000000000000ULL;
+        const bool has = use && hi < 0x7ff00000u;   // finite, not negative
+        const unsigned long long key = has ? (unsigned long long)hi << 32 | lo : 0x7ff0000000000000ULL;
         const unsigned long long k0 = __shfl_sync(FULL, key, base), k1 = __shfl_sync(FULL, key, base + 1),
                                  k2 = __shfl_sync(FULL, key, base + 2);
         int ax = -1;
@@ -1021,7 +1032,17 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
         if (k0 < km) { km = k0; ax = 0; }
         if (k1 < km) { km = k1; ax = 1; }
         if (k2 < km) { km = k2; ax = 2; }
-        const double tmin = __longlong_as_double((long long)km);
+        double tmin = __longlong_as_double((long long)km);
+        if constexpr (EXACT) {   // the general choice, negative times (offsets outside the cell) among them
+            const double t = use && hi_abs(hi) < 0x7ff00000u ? te : CUDART_INF;
+            const double t0 = __shfl_sync(FULL, t, base), t1 = __shfl_sync(FULL, t, base + 1),
+                         t2 = __shfl_sync(FULL, t, base + 2);
+            ax = -1;
+            tmin = CUDART_INF;
+            if (t0 < tmin) { tmin = t0; ax = 0; }
+            if (t1 < tmin) { tmin = t1; ax = 1; }
+            if (t2 < tmin) { tmin = t2; ax = 2; }
+        }
         const int fx = ax < 0 ? 0 : ((up >> (base + ax)) & 1u) ? 1 : -1;
         const int fidx = 2 * ax + (fx > 0 ? 1 : 0);
         // the neighbour across the exit face, read while the axes move
@@ -1037,16 +1058,13 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
         again = again && a != ax;
         // an event: an output time or the stop time in the step, no exit, a
         // path that ends here, the step cap, a motion for the general form, a
-        // candidate whose exact time is not finite: if that is the leading
-        // one, the others' times are not bounded by it, so every reachable
-        // axis decides, as in the one-lane engine
-        const bool open = use && !has && !exact && em >= 0.0f;
+        // candidate whose exact time is not finite (if that is the leading
+        // one, the others' times are not bounded by it) or is negative: then
+        // every reachable axis decides, as in the one-lane engine
+        const bool open = !EXACT && use && !has;
         const bool ev = go && (ax < 0 || tkey(t_end) >= s.tev);
         if (__any_sync(FULL, open || ev || (live && (!go || !enter || again)))) {
-            if (__any_sync(FULL, open)) {
-                exact = true;
-                continue;
-            }
+            if (!EXACT && __any_sync(FULL, open)) return false;
             enum { P_NONE, P_CROSS, P_TIME, P_NOEXIT, P_CAPTURE };
             int path = go ? P_CROSS : P_NONE, m = 0;
             if (ev) {   // (the stop time is never before tev)
@@ -1095,7 +1113,6 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
                 going = __any_sync(FULL, live);
             }
         }
-        exact = false;
         if (go && live) {
             // hand over to the neighbour; the exit coordinate enters on the shared face
             s.steps++;
@@ -1112,7 +1129,10 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
             gather_axes(s, x, ix, base);
             pl_push(e, P, pcount, s, q, lead && go && live && p.pathline, s.st);
         }
-    }
+        return true;
+    };
+    while (going)
+        if (!step(std::false_type{})) step(std::true_type{});
     if (TS) rec_finish(e, Q, qcount);
     if (PL) pl_flush(e, P, pcount);
     flush_counters(e, s_cnt);
