@@ -258,6 +258,10 @@ const char* mp_last_error(void);
  * per-cell velocity records in FP64 and FP32 (the paper's central flow-data
  * object, Methods, "Multiprocessing"), neighbour classes and face
  * coordinates.  Validates shapes, finiteness and porosity.  Synchronous.
+ * Device arrays (MP_DEVICE_PTR) are read after the work enqueued before the
+ * call on the legacy default stream and on blocking streams; what writes them
+ * on a non-blocking stream (cudaStreamNonBlocking) has to be complete, or the
+ * default stream made to wait for it, before the call.
  * Errors: MP_ERR_INVALID_ARG, MP_ERR_SHAPE, MP_ERR_NONFINITE, MP_ERR_OOM,
  * MP_ERR_CUDA. */
 /* Passage: Methods, "MODPATH" (the tracking reads the flow model's cell data) and

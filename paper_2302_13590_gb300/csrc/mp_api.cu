@@ -153,6 +153,7 @@ struct mp_ctx {
     std::mutex host_mu;                             // one mp_track_host at a time per context
     cudaStream_t host_st[3] = {nullptr, nullptr, nullptr};   // its streams (two that track, one that copies back)
     cudaStream_t load_st = nullptr;                 // field loads and frees
+    cudaEvent_t load_ev = nullptr;                  // what a load's device arrays wait for
     cudaMemPool_t field_pool = nullptr;             // fields and their load's scratch
     std::map<TuneKey, mp_tuning> tuned;
     std::map<int64_t, Request*> reqs;
@@ -272,6 +273,7 @@ int mp_ctx_create(int device, mp_ctx** out)
     props.location.type = cudaMemLocationTypeDevice;
     props.location.id = device;
     cudaError_t e = cudaStreamCreateWithFlags(&c->load_st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->load_ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemPoolCreate(&c->field_pool, &props);
     if (e == cudaSuccess) {
         uint64_t keep = FIELD_POOL_KEEP;
@@ -279,6 +281,7 @@ int mp_ctx_create(int device, mp_ctx** out)
     }
     if (e != cudaSuccess) {
         if (c->field_pool) cudaMemPoolDestroy(c->field_pool);
+        if (c->load_ev) cudaEventDestroy(c->load_ev);
         if (c->load_st) cudaStreamDestroy(c->load_st);
         delete c;
         return cuda_fail(e, "mp_ctx_create: field pool");
@@ -307,6 +310,7 @@ int mp_ctx_destroy(mp_ctx* ctx)
     for (cudaStream_t x : ctx->host_st)
         if (x) cudaStreamDestroy(x);
     cudaStreamDestroy(ctx->load_st);
+    cudaEventDestroy(ctx->load_ev);
     cudaMemPoolDestroy(ctx->field_pool);
     delete ctx;
     return MP_OK;
@@ -403,7 +407,16 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     const double* qz = dev_in ? d->qz : reinterpret_cast<double*>(stage + o_qz);
     const double* por = dev_in ? d->porosity : reinterpret_cast<double*>(stage + o_por);
     cudaError_t e = cudaSuccess;
-    if (!dev_in) {
+    if (dev_in) {
+        // The caller's arrays are read on a stream of the context's own, so
+        // they wait for the work that may still write them: the default
+        // stream's, and with it every blocking stream's (1.6 us; a wait for
+        // the device would reach the others too, but breaks a capture that
+        // another thread has under way).
+        if ((e = cudaEventRecord(ctx->load_ev, cudaStreamLegacy)) != cudaSuccess ||
+            (e = cudaStreamWaitEvent(s, ctx->load_ev, 0)) != cudaSuccess)
+            return fin(cuda_fail(e, "mp_field_load: order"));
+    } else {
         if ((e = cudaMemcpyAsync(stage + o_qx, d->qx, sizeof(double) * nqx, h2d, s)) != cudaSuccess ||
             (e = cudaMemcpyAsync(stage + o_qy, d->qy, sizeof(double) * nqy, h2d, s)) != cudaSuccess ||
             (e = cudaMemcpyAsync(stage + o_qz, d->qz, sizeof(double) * nqz, h2d, s)) != cudaSuccess ||

@@ -212,6 +212,15 @@ def _stream(s):
 
 # ---- C-named functions ----------------------------------------------------------
 
+def _finish_current_stream(t):
+    """Wait for torch's current stream on t's device.  The library orders a
+    load after the default stream; torch's other streams are non-blocking."""
+    import torch
+    s = torch.cuda.current_stream(t.device)
+    if s.cuda_stream != 0 and not torch.cuda.is_current_stream_capturing():   # (0: the default stream)
+        s.synchronize()
+
+
 def mp_ctx_create(device: int = 0):
     h = ctypes.c_void_p()
     _check(load_library().mp_ctx_create(int(device), ctypes.byref(h)))
@@ -225,12 +234,14 @@ def mp_ctx_destroy(ctx):
 def mp_field_load(ctx, field, device_arrays: bool = False):
     """Load a field (an object with nlay, nrow, ncol, delr, delc, dz, origin,
     qx, qy, qz, porosity, ibound).  With device_arrays=True the flow arrays are
-    CUDA tensors (float64 / int8, contiguous) read in place."""
+    CUDA tensors (float64 / int8, contiguous) read in place, after what is
+    enqueued on torch's current stream and on the default stream."""
     keep = []
     delr, delc, dz = (_host(field.delr, np.float64), _host(field.delc, np.float64), _host(field.dz, np.float64))
     keep += [delr, delc, dz]
     if device_arrays:
         arrs = [field.qx, field.qy, field.qz, field.porosity, field.ibound]
+        _finish_current_stream(arrs[0])
     else:
         arrs = [_host(field.qx, np.float64), _host(field.qy, np.float64), _host(field.qz, np.float64),
                 _host(field.porosity, np.float64), _host(field.ibound, np.int8)]
