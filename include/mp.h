@@ -267,6 +267,11 @@ const char* mp_last_error(void);
 /* Passage: Methods, "MODPATH" (the tracking reads the flow model's cell data) and
  * "Multiprocessing" (flow-related arrays stored once, centrally, reached through a pointer). */
 int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out);
+/* Waits (bounded) for the requests that read the field and still have their
+ * ids; work that no id stands for any more (a freed request, a release, an
+ * mp_track_noalloc that did not wait) may still be running: the memory is
+ * handed on behind it.  May be called while another stream is captured.
+ * Errors: MP_ERR_INVALID_ARG, MP_ERR_TIMEOUT (then nothing is freed). */
 /* Passage: none (infrastructure). */
 int mp_field_free(mp_field* f);
 

@@ -6,6 +6,7 @@
 // Request outputs come from the stream-ordered allocator so that many
 // requests can be admitted, run and released without device-wide syncs.
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -107,6 +108,9 @@ struct mp_field {
     DevUsg u{};
     void* buf = nullptr;   // one allocation for all device arrays
     size_t bytes = 0;
+    mutable std::atomic<bool> foreign{false};     // work on it that the context has no events of (another context's)
+    cudaEvent_t na_ev = nullptr;                  // end of the last mp_track_noalloc that did not wait
+    mutable std::atomic<bool> na_used{false};     // na_ev is recorded
     std::vector<double> geom;   // dims, delr, delc, dz, origin: fields with equal geom share a grid
 };
 
@@ -118,9 +122,15 @@ struct mp_group {
     size_t bytes = 0;
     long long n = 0;
     cudaStream_t stream = nullptr;
+    // the release: the field it reads, its stream's id, and whether a request
+    // on that field and stream follows it (whose end then stands for both)
+    const mp_field* released_on = nullptr;
+    unsigned long long sid = 0;
+    bool covered = false;
 };
 
 struct Request {
+    mp_ctx* ctx = nullptr;
     mp_group* group = nullptr;
     std::vector<const mp_field*> fields;   // every field its launches read
     long long n = 0;
@@ -132,6 +142,8 @@ struct Request {
     unsigned long long* queue = nullptr;   // queue head of its own launches, in buf after the counters
     cudaStream_t stream = nullptr;
     cudaEvent_t k0 = nullptr, k1 = nullptr;
+    unsigned long long sid = 0, seq = 0;   // id of the stream that k1 was recorded on, order of the recording
+    bool captured = false;      // recorded into a capture of the caller's
     bool graph_owned = false;   // outputs of a captured graph: freed with it, events shared
 };
 
@@ -152,7 +164,8 @@ struct mp_ctx {
     std::mutex mu;
     std::mutex host_mu;                             // one mp_track_host at a time per context
     cudaStream_t host_st[3] = {nullptr, nullptr, nullptr};   // its streams (two that track, one that copies back)
-    cudaStream_t load_st = nullptr;                 // field loads and frees
+    cudaStream_t load_st = nullptr;                 // field loads and frees (one stream: the pool hands a freed
+                                                    // field's memory to the next load in its order)
     cudaEvent_t load_ev = nullptr;                  // what a load's device arrays wait for
     cudaMemPool_t field_pool = nullptr;             // fields and their load's scratch
     std::map<TuneKey, mp_tuning> tuned;
@@ -161,9 +174,48 @@ struct mp_ctx {
     std::set<mp_group*> groups;
     std::set<mp_graph*> graphs;
     int64_t next_id = 1;
+    // Per stream (by its id, which no later stream takes over) the end of the
+    // last work on it whose request or group is gone.
+    struct End {
+        unsigned long long seq;
+        cudaEvent_t ev;
+    };
+    std::map<unsigned long long, End> ended;
+    unsigned long long next_seq = 1;
 };
 
 namespace {
+
+// Keep ev (recorded as number seq on stream sid) for the fields freed later;
+// of one stream's events only the last matters.  ctx->mu is held.
+void keep_end(mp_ctx* ctx, unsigned long long sid, unsigned long long seq, cudaEvent_t ev)
+{
+    if (ctx->ended.size() > 64) {   // streams come and go: forget what is over
+        for (auto it = ctx->ended.begin(); it != ctx->ended.end();) {
+            if (cudaEventQuery(it->second.ev) == cudaSuccess) {
+                cudaEventDestroy(it->second.ev);
+                it = ctx->ended.erase(it);
+            } else {
+                ++it;
+            }
+        }
+    }
+    mp_ctx::End& x = ctx->ended[sid];   // (a new entry: seq 0)
+    if (seq > x.seq) std::swap(ev, x.ev), x.seq = seq;
+    if (ev) cudaEventDestroy(ev);
+}
+
+// The device's work so far, with any stream: what cudaFree does, also while
+// another stream is captured (cudaDeviceSynchronize would break the capture).
+// 65 us, so only where the events do not tell.
+cudaError_t device_wait()
+{
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, 256);
+    if (e == cudaSuccess) return cudaFree(p);
+    cudaGetLastError();
+    return cudaDeviceSynchronize();
+}
 
 // Wait (bounded) until no request of ctx still reads the given group/field.
 int drain_users(mp_ctx* ctx, const mp_group* g, const mp_field* f)
@@ -309,6 +361,7 @@ int mp_ctx_destroy(mp_ctx* ctx)
     cudaDeviceSynchronize();
     for (cudaStream_t x : ctx->host_st)
         if (x) cudaStreamDestroy(x);
+    for (auto& x : ctx->ended) cudaEventDestroy(x.second.ev);
     cudaStreamDestroy(ctx->load_st);
     cudaEventDestroy(ctx->load_ev);
     cudaMemPoolDestroy(ctx->field_pool);
@@ -462,12 +515,15 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     if (got.flags & 2u) return fin(fail(MP_ERR_NONFINITE, "mp_field_load: porosity outside (0, 1] in an active cell"));
     if (got.flags & 4u) return fin(fail(MP_ERR_INVALID_ARG, "mp_field_load: ibound outside {-1, 0, 1, 2}"));
     mp_balance bal{};
-    if ((e = balance_report(ctx, got.total, dio, ncell, parts, &bal)) != cudaSuccess)
+    cudaEvent_t na_ev = nullptr;   // (made here: mp_track_noalloc allocates nothing)
+    if ((e = balance_report(ctx, got.total, dio, ncell, parts, &bal)) != cudaSuccess ||
+        (e = cudaEventCreateWithFlags(&na_ev, cudaEventDisableTiming)) != cudaSuccess)
         return fin(cuda_fail(e, "mp_field_load: balance"));
     cudaFreeAsync(stage, s);
 
     mp_field* f = new mp_field();
     f->ctx = ctx;
+    f->na_ev = na_ev;
     f->d = v;
     f->balance = bal;
     f->buf = buf;
@@ -494,15 +550,40 @@ int mp_field_free(mp_field* f)
     mp_ctx* ctx = f->ctx;
     int rc = drain_users(ctx, nullptr, f);
     if (rc != MP_OK) return rc;
-    // every stream's work first (a release or an allocation-free launch may
-    // still read the field): the memory is handed on in load_st's order
     cudaSetDevice(ctx->device);
-    MP_CUDA(cudaDeviceSynchronize(), "mp_field_free");
+    // The memory goes back behind everything that may still read the field:
+    // requests and groups that are gone, releases on it, a launch without
+    // allocation.  load_st waits for them, this thread and the device do not.
+    cudaError_t e = cudaSuccess;
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
+        for (mp_group* g : ctx->groups) {
+            if (g->released_on != f) continue;
+            g->released_on = nullptr;
+            if (g->covered || e != cudaSuccess) continue;
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            cudaEvent_t ev = nullptr;
+            e = cudaStreamIsCapturing(g->stream, &cap);
+            if (e == cudaSuccess && cap != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventRecord(ev, g->stream);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->load_st, ev, 0);
+            if (ev) cudaEventDestroy(ev);
+        }
+        for (auto& x : ctx->ended) {
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->load_st, x.second.ev, 0);
+            cudaEventDestroy(x.second.ev);
+        }
+        ctx->ended.clear();
         ctx->fields.erase(f);
     }
+    if (e == cudaSuccess && f->na_used) e = cudaStreamWaitEvent(ctx->load_st, f->na_ev, 0);
+    if (e != cudaSuccess || f->foreign) {
+        cudaGetLastError();
+        device_wait();
+    }
     cudaFreeAsync(f->buf, ctx->load_st);
+    if (f->na_ev) cudaEventDestroy(f->na_ev);
     delete f;
     return MP_OK;
 }
@@ -674,6 +755,9 @@ int mp_release_group(mp_ctx* ctx, const mp_field* f, const mp_release_desc* r, v
     g->buf = buf;
     g->bytes = bytes;
     g->stream = s;
+    g->released_on = f;
+    cudaStreamGetId(s, &g->sid);
+    if (f->ctx != ctx) f->foreign = true;
     g->d = group_view(buf, n);
     // a fresh particle: no steps yet (hash and exit face are read only after one)
     if (f->usg && r->kind == MP_RELEASE_BOX) {
@@ -728,11 +812,25 @@ int mp_group_free(mp_group* g)
     mp_ctx* ctx = g->ctx;
     int rc = drain_users(ctx, g, nullptr);
     if (rc != MP_OK) return rc;
+    cudaSetDevice(ctx->device);
     {
         std::lock_guard<std::mutex> lk(ctx->mu);
         ctx->groups.erase(g);
+        if (!g->covered && ctx->fields.count(const_cast<mp_field*>(g->released_on))) {
+            // the release may still run
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            cudaEvent_t ev = nullptr;
+            if (cudaStreamIsCapturing(g->stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+                cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&
+                cudaEventRecord(ev, g->stream) == cudaSuccess) {
+                keep_end(ctx, g->sid, ctx->next_seq++, ev);
+            } else {
+                cudaGetLastError();
+                if (ev) cudaEventDestroy(ev);
+                g->released_on->foreign = true;   // no event tells: its free waits for the device
+            }
+        }
     }
-    cudaSetDevice(ctx->device);
     cudaFreeAsync(g->buf, g->stream);
     delete g;
     return MP_OK;
@@ -848,6 +946,8 @@ int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream
         return fail(MP_ERR_OOM, "mp_track: device allocation failed");
     }
     Request* r = new Request();
+    r->ctx = ctx;
+    if (g->field->ctx != ctx) g->field->foreign = true;
     r->group = g;
     r->fields.push_back(g->field);
     r->n = n;
@@ -934,6 +1034,20 @@ void drop_request(Request* r)
     delete r;
 }
 
+// a launched request that nobody waited for: its end is kept
+void end_request(Request* r)
+{
+    cudaFreeAsync(r->buf, r->stream);
+    cudaEventDestroy(r->k0);
+    if (r->captured) {
+        cudaEventDestroy(r->k1);
+    } else {
+        std::lock_guard<std::mutex> lk(r->ctx->mu);
+        keep_end(r->ctx, r->sid, r->seq, r->k1);
+    }
+    delete r;
+}
+
 // One launch over prepared requests of one precision (Methods,
 // "Multiprocessing": a single particle loop over every particle).
 // ev: 1 records the requests' start events before the launch, 2 their end
@@ -1000,7 +1114,23 @@ int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, const
                                                 : launch_track_mixed_f64t(fd, b, modes, schedule, block, s);
         if (e == cudaSuccess) e = mp::launch_spread_window(b, s);
     }
-    for (int i = 0; i < n && e == cudaSuccess && (ev & 2u); ++i) e = cudaEventRecord(rs[i]->k1, s);
+    if (e == cudaSuccess && (ev & 2u)) {
+        unsigned long long sid = 0;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const bool plain = cudaStreamGetId(s, &sid) == cudaSuccess && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+                           cap == cudaStreamCaptureStatusNone;
+        std::lock_guard<std::mutex> lk(rs[0]->ctx->mu);   // (the numbers follow the order of the recordings)
+        for (int i = 0; i < n && e == cudaSuccess; ++i) {
+            Request* r = rs[i];
+            e = cudaEventRecord(r->k1, s);
+            r->sid = sid;
+            r->seq = r->ctx->next_seq++;
+            r->captured = !plain;
+            mp_group* g = r->group;
+            if (g->sid == sid && plain && std::find(r->fields.begin(), r->fields.end(), g->released_on) != r->fields.end())
+                g->covered = true;
+        }
+    }
     if (tbl) cudaFreeAsync(tbl, s);
     if (e != cudaSuccess) return cuda_fail(e, "mp_track: launch");
     return MP_OK;
@@ -1402,10 +1532,7 @@ int mp_req_free(mp_ctx* ctx, mp_req id)
         ctx->reqs.erase(it);
     }
     cudaSetDevice(ctx->device);
-    cudaFreeAsync(r->buf, r->stream);
-    cudaEventDestroy(r->k0);
-    cudaEventDestroy(r->k1);
-    delete r;
+    end_request(r);
     return MP_OK;
 }
 
@@ -1547,6 +1674,12 @@ void set_last_error(const char* msg) { g_err = msg ? msg : ""; }
 const DevField* field_device_view(const mp_field* f) { return &f->d; }
 bool field_is_usg(const mp_field* f) { return f->usg != 0; }
 int field_device(const mp_field* f) { return f->ctx->device; }
+cudaError_t field_used(const mp_field* f, cudaStream_t s)
+{
+    const cudaError_t e = cudaEventRecord(f->na_ev, s);
+    f->na_used = true;
+    return e;
+}
 
 }  // namespace mp
 
@@ -1592,7 +1725,8 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
         if (rc == MP_OK) rc = wait_event(r->k1, -1);
         float ms = 0.f;
         if (rc == MP_OK && cudaEventElapsedTime(&ms, r->k0, r->k1) != cudaSuccess) rc = fail(MP_ERR_CUDA, "timing");
-        drop_request(r);
+        if (r->seq) end_request(r);
+        else drop_request(r);
         if (rc != MP_OK) return rc;
         if (ci > 0 && ms < best.ms) {
             best.ms = ms;

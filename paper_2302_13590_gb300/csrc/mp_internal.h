@@ -326,5 +326,7 @@ void set_last_error(const char* msg);
 const DevField* field_device_view(const mp_field* f);
 bool field_is_usg(const mp_field* f);
 int field_device(const mp_field* f);   // the device of the field's context
+// a launch on s that no request stands for reads the field: its memory is handed on after it
+cudaError_t field_used(const mp_field* f, cudaStream_t s);
 
 }  // namespace mp

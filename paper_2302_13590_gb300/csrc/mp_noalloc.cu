@@ -146,7 +146,10 @@ int track_noalloc(const mp_field* f, const mp_noalloc_args* a, cudaStream_t s, m
     e = (o->precision == MP_PREC_FP64) ? launch_track_fp64(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, o->block, s)
                                        : launch_track_mixed(fd, b, nt > 0 ? MODE_TS : 0u, o->schedule, o->block, s);
     if (e != cudaSuccess) return na_fail(MP_ERR_CUDA, std::string("mp_track_noalloc: launch: ") + cudaGetErrorString(e));
-    if (stats) {
+    if (!stats) {
+        e = mp::field_used(f, s);
+        if (e != cudaSuccess) return na_fail(MP_ERR_CUDA, std::string("mp_track_noalloc: ") + cudaGetErrorString(e));
+    } else {
         unsigned long long h[N_COUNTERS];
         e = cudaMemcpyAsync(h, counters, sizeof(h), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
