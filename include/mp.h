@@ -271,6 +271,9 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out);
  * ids; work that no id stands for any more (a freed request, a release, an
  * mp_track_noalloc that did not wait) may still be running: the memory is
  * handed on behind it.  May be called while another stream is captured.
+ * The context keeps up to 1 GiB of freed fields' memory for its next loads;
+ * it goes back with the context, or when an allocation of the library (of any
+ * context on the device) would fail without it.
  * Errors: MP_ERR_INVALID_ARG, MP_ERR_TIMEOUT (then nothing is freed). */
 /* Passage: none (infrastructure). */
 int mp_field_free(mp_field* f);

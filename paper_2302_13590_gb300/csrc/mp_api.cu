@@ -205,6 +205,51 @@ void keep_end(mp_ctx* ctx, unsigned long long sid, unsigned long long seq, cudaE
     if (ev) cudaEventDestroy(ev);
 }
 
+// Every context of the process, for give_back.
+std::mutex g_ctx_mu;
+std::set<mp_ctx*> g_ctx;
+
+// Memory of freed fields that the contexts on a device keep, to the device
+// (behind a bounded wait for the frees that are still to run).
+void give_back(int device)
+{
+    std::lock_guard<std::mutex> lk(g_ctx_mu);
+    for (mp_ctx* c : g_ctx) {
+        if (c->device != device) continue;
+        cudaEvent_t ev = nullptr;
+        if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess &&
+            cudaEventRecord(ev, c->load_st) == cudaSuccess && wait_event(ev, -1) == MP_OK &&
+            cudaEventSynchronize(ev) == cudaSuccess)   // (over; but the pool learns of its frees by a synchronisation)
+            cudaMemPoolTrimTo(c->field_pool, 0);
+        if (ev) cudaEventDestroy(ev);
+    }
+    cudaMemPool_t pool;   // and what the requests' pool does not use
+    if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+    cudaGetLastError();
+}
+
+// An allocation that is refused for want of memory is tried again once the
+// kept memory has gone back: a context takes no less than what is there.
+template <class A>
+cudaError_t alloc_or_give_back(const mp_ctx* ctx, A&& alloc)
+{
+    cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    give_back(ctx->device);
+    return alloc();
+}
+template <class T>
+cudaError_t pool_alloc(const mp_ctx* ctx, T** p, size_t bytes, cudaStream_t s)   // requests and groups
+{
+    return alloc_or_give_back(ctx, [&] { return cudaMallocAsync(p, bytes, s); });
+}
+template <class T>
+cudaError_t field_alloc(const mp_ctx* ctx, T** p, size_t bytes)   // fields, on load_st
+{
+    return alloc_or_give_back(ctx, [&] { return cudaMallocFromPoolAsync(p, bytes, ctx->field_pool, ctx->load_st); });
+}
+
 // The device's work so far, with any stream: what cudaFree does, also while
 // another stream is captured (cudaDeviceSynchronize would break the capture).
 // 65 us, so only where the events do not tell.
@@ -255,7 +300,8 @@ int read_counters(Request* r, unsigned long long* h)
 // this much when fields are freed: the next load of a transient model's field
 // then reuses mapped memory (cudaMalloc and cudaFree of a 200x200x20 field's
 // 136 MB took 1.1 ms).  What is above goes back at the next synchronisation,
-// the rest with the context.
+// the rest with the context, or when an allocation of the library would fail
+// without it (give_back).
 constexpr uint64_t FIELD_POOL_KEEP = 1ULL << 30;
 
 // the report of a reduced balance; the sink cells' extractions are read and
@@ -278,7 +324,7 @@ cudaError_t balance_report(mp_ctx* ctx, const BalancePart& t, const double2* ino
         const cudaStream_t s = ctx->load_st;
         std::vector<double> x((size_t)t.sinks);
         double* packed = nullptr;
-        cudaError_t e = cudaMallocFromPoolAsync(&packed, sizeof(double) * x.size(), ctx->field_pool, s);
+        cudaError_t e = field_alloc(ctx, &packed, sizeof(double) * x.size());
         if (e != cudaSuccess) return e;
         e = launch_balance_sinks(inout, ncell, parts, packed, s);
         if (e == cudaSuccess)
@@ -338,6 +384,10 @@ int mp_ctx_create(int device, mp_ctx** out)
         delete c;
         return cuda_fail(e, "mp_ctx_create: field pool");
     }
+    {
+        std::lock_guard<std::mutex> lk(g_ctx_mu);
+        g_ctx.insert(c);
+    }
     *out = c;
     return MP_OK;
 }
@@ -346,6 +396,10 @@ int mp_ctx_destroy(mp_ctx* ctx)
 {
     if (!ctx) return fail(MP_ERR_INVALID_ARG, "mp_ctx_destroy: NULL");
     cudaSetDevice(ctx->device);
+    {
+        std::lock_guard<std::mutex> lk(g_ctx_mu);
+        g_ctx.erase(ctx);
+    }
     std::vector<mp_graph*> grs(ctx->graphs.begin(), ctx->graphs.end());
     for (mp_graph* g : grs) mp_graph_free(g);
     std::vector<mp_req> ids;
@@ -420,8 +474,7 @@ int mp_field_load(mp_ctx* ctx, const mp_field_desc* d, mp_field** out)
     const cudaStream_t s = ctx->load_st;
     char* buf = nullptr;
     char* stage = nullptr;
-    if (cudaMallocFromPoolAsync(&buf, persistent, ctx->field_pool, s) != cudaSuccess ||
-        cudaMallocFromPoolAsync(&stage, soff, ctx->field_pool, s) != cudaSuccess) {
+    if (field_alloc(ctx, &buf, persistent) != cudaSuccess || field_alloc(ctx, &stage, soff) != cudaSuccess) {
         cudaGetLastError();
         if (buf) cudaFreeAsync(buf, s);
         return fail(MP_ERR_OOM, "mp_field_load: device allocation failed");
@@ -636,8 +689,7 @@ int mp_usg_field_load(mp_ctx* ctx, const mp_usg_desc* d, mp_field** out)
     const cudaStream_t s = ctx->load_st;
     char* buf = nullptr;
     char* stage = nullptr;
-    if (cudaMallocFromPoolAsync(&buf, persistent, ctx->field_pool, s) != cudaSuccess ||
-        cudaMallocFromPoolAsync(&stage, soff, ctx->field_pool, s) != cudaSuccess) {
+    if (field_alloc(ctx, &buf, persistent) != cudaSuccess || field_alloc(ctx, &stage, soff) != cudaSuccess) {
         cudaGetLastError();
         if (buf) cudaFreeAsync(buf, s);
         return fail(MP_ERR_OOM, "mp_usg_field_load: device allocation failed");
@@ -744,7 +796,7 @@ int mp_release_group(mp_ctx* ctx, const mp_field* f, const mp_release_desc* r, v
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const size_t bytes = group_bytes(n);
     char* buf = nullptr;
-    if (cudaMallocAsync(&buf, bytes, s) != cudaSuccess) {
+    if (pool_alloc(ctx, &buf, bytes, s) != cudaSuccess) {
         cudaGetLastError();
         return fail(MP_ERR_OOM, "mp_release_group: device allocation failed");
     }
@@ -779,7 +831,7 @@ int mp_release_group(mp_ctx* ctx, const mp_field* f, const mp_release_desc* r, v
             const size_t o_c = toff; toff = align256(toff + 4 * (size_t)n);
             const size_t o_l = toff; toff = align256(toff + 24 * (size_t)n);
             const size_t o_t0 = toff; toff = align256(toff + (r->t0 ? 8 * (size_t)n : 0));
-            e = cudaMallocAsync(&tmp, toff, s);
+            e = pool_alloc(ctx, &tmp, toff, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(tmp + o_c, r->cell, 4 * (size_t)n, cudaMemcpyHostToDevice, s);
             if (e == cudaSuccess) e = cudaMemcpyAsync(tmp + o_l, r->local, 24 * (size_t)n, cudaMemcpyHostToDevice, s);
             if (e == cudaSuccess && r->t0)
@@ -941,7 +993,7 @@ int prepare_request(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, cudaStream
     oo.n_times = nt;
     mp_query_bytes(&oo, n, &bytes);
     char* buf = nullptr;
-    if (cudaMallocAsync(&buf, std::max<size_t>(bytes, 256), s) != cudaSuccess) {
+    if (pool_alloc(ctx, &buf, std::max<size_t>(bytes, 256), s) != cudaSuccess) {
         cudaGetLastError();
         return fail(MP_ERR_OOM, "mp_track: device allocation failed");
     }
@@ -1082,7 +1134,7 @@ int launch_requests(const mp_field* f, Request** rs, const mp::Req* hreqs, const
             o_t[i] = again ? o_t[i - 1] : off;
             if (!again) off = align256(off + times_bytes(hreqs[i].p.n_times));
         }
-        if (cudaMallocAsync(&tbl, off, s) != cudaSuccess) {
+        if (pool_alloc(rs[0]->ctx, &tbl, off, s) != cudaSuccess) {
             cudaGetLastError();
             return fail(MP_ERR_OOM, "mp_track: device allocation failed");
         }
@@ -1298,7 +1350,7 @@ int mp_track_periods(mp_ctx* ctx, mp_group* g, int n_periods, const mp_field* co
     r->fields.assign(fields, fields + n_periods);
     // the periods advance a request-owned copy of the group's state
     char* scratch = nullptr;
-    if (cudaMallocAsync(&scratch, g->bytes, s) != cudaSuccess) {
+    if (pool_alloc(ctx, &scratch, g->bytes, s) != cudaSuccess) {
         cudaGetLastError();
         drop_request(r);
         return fail(MP_ERR_OOM, "mp_track_periods: device allocation failed");
@@ -1819,7 +1871,7 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
     // group state of every request in one allocation
     std::vector<size_t> goff((size_t)n_reqs + 1, 0);
     for (int i = 0; i < n_reqs; ++i) goff[i + 1] = goff[i] + align256(group_bytes(rel[i].n));
-    if (cudaMalloc(&G->state, goff[n_reqs]) != cudaSuccess) {
+    if (alloc_or_give_back(ctx, [&] { return cudaMalloc(&G->state, goff[n_reqs]); }) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(MP_ERR_OOM, "mp_graph_create: device allocation failed"));
     }
@@ -1869,7 +1921,7 @@ int mp_graph_create(mp_ctx* ctx, const mp_field* f, int n_reqs, const mp_release
         o_bst[p] = off; off = align256(off + sizeof(long long) * (sel[p].size() + 1));
         o_q[p] = off; off = align256(off + sizeof(unsigned long long));
     }
-    if (cudaMalloc(&G->tables, off) != cudaSuccess) {
+    if (alloc_or_give_back(ctx, [&] { return cudaMalloc(&G->tables, off); }) != cudaSuccess) {
         cudaGetLastError();
         return bail(fail(MP_ERR_OOM, "mp_graph_create: device allocation failed"));
     }
