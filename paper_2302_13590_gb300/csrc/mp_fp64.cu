@@ -1049,7 +1049,9 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
         const int cls = ax < 0 ? (int)NB_OUTSIDE : (int)((c.nb >> (2 * fidx)) & 3u);
         const int c2 = s.c + fx * (ax == 0 ? 1 : (ax == 1 ? stride_y : stride_z));
         const int ix2 = ix + (a == ax ? fx : 0);
-        const bool enter = go && ax >= 0 && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
+        const bool inside = (unsigned)c2 < (unsigned)f.ncell;   // (false across an outer face; else an error)
+        const bool enter =
+            go && ax >= 0 && inside && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
         AxisRec n = c;
         if (enter) n = read_axis(f, c2, a, axis_at + ix2);
         const double t_end = s.t + tmin;
@@ -1094,6 +1096,10 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
                     s.t = t_end;
                     s.ef = fidx;
                     s.st = cls == NB_OUTSIDE ? MP_ST_EXIT_DOMAIN : (cls == NB_BOUNDARY ? MP_ST_BOUNDARY : MP_ST_SINK);
+                    if (!inside && (cls == NB_ACTIVE || cls == NB_SINK)) {
+                        if (lead) atomicCAS(e.req(s.r).o.counters + COUNTER_ERR, 0ULL, (unsigned long long)q + 1ULL);
+                        s.st = MP_ST_INVALID_RELEASE;
+                    }
                 }
             } else if (path == P_TIME) {
                 x = f64_move(c.A, c.iA, c.D, vp, x, p.t_stop - s.t);

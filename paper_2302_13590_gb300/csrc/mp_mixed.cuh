@@ -639,7 +639,9 @@ __global__ void __launch_bounds__(32) k_track_axes_mixed(MixEngine<false, ONE> e
         const int fidx = 2 * ax + (fx > 0 ? 1 : 0);
         const int cls = ax < 0 ? (int)NB_OUTSIDE : (int)((nb >> (2 * fidx)) & 3u);
         const int c2 = s.c + fx * (ax == 0 ? 1 : (ax == 1 ? stride_y : stride_z));
-        const bool enter = go && ax >= 0 && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
+        const bool inside = (unsigned)c2 < (unsigned)f.ncell;   // (false across an outer face; else an error)
+        const bool enter =
+            go && ax >= 0 && inside && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
         float n1 = 0.0f, n2 = 0.0f;
         unsigned nnb = 0;
         if (enter) read(c2, n1, n2, nnb);
@@ -694,6 +696,10 @@ __global__ void __launch_bounds__(32) k_track_axes_mixed(MixEngine<false, ONE> e
                 s.tl = nl;
                 s.ef = fidx;
                 s.st = cls == NB_OUTSIDE ? MP_ST_EXIT_DOMAIN : (cls == NB_BOUNDARY ? MP_ST_BOUNDARY : MP_ST_SINK);
+                if (!inside && (cls == NB_ACTIVE || cls == NB_SINK)) {
+                    if (lead) atomicCAS(e.req(s.r).o.counters + COUNTER_ERR, 0ULL, (unsigned long long)q + 1ULL);
+                    s.st = MP_ST_INVALID_RELEASE;
+                }
             } else if (path == P_TIME) {
                 x = E::move(A, up, x, E::ff_diff(p.tstop_hi, p.tstop_lo, s.th, s.tl));
                 s.th = p.tstop_hi;
