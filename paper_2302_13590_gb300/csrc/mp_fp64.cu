@@ -986,6 +986,7 @@ __global__ void __launch_bounds__(32) k_track_axes(F64Engine<ONE> e)
     if (PL)
         pl_push(e, P, pcount, s, q, lead && loaded && path_start(e, s), s.st == MP_ST_TIME ? MP_ST_ACTIVE : s.st);
     if (TS) tail_fill(e, s, q, lead && ended && !paused(e, s));
+    __syncwarp();   // finish may write the group's state, which the group's other lanes load too
     if (lead && ended) e.template finish<TS>(q, s, s_cnt);
     // this lane's axis: offset and index, and the cell's record of it
     double x = a == 0 ? s.x0 : (a == 1 ? s.x1 : s.x2);
