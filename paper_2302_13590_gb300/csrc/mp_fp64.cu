@@ -913,12 +913,12 @@ struct F64Engine {
 // the same.  One step of 4864 particles 2.7 -> 1.7 us; 1000 particles, 50x50
 // cells 135 -> 93 us; 5003 pathlines, 7x61x83 cells 449 -> 277 us; 10,000
 // particles to a stop time, 200x200x20 cells 772 -> 491 us.
-// Launches of up to this many particles take three lanes each: 12 warps an SM
-// (three a sub-partition) on 152 SMs.  There both forms are FP64 bound at
-// about the same time (endpoints, 200x200x20 cells, 329 steps the longest:
-// 4864 particles 550 us against 880, 9728: 629 / 947, 19456: 1020 / 979,
-// 38912: 2317 / 1050).
-constexpr long long AXES_MAX = 12 * 152 * AXES_PARTICLES;
+// Launches of up to this many warps of ten particles on each SM take three
+// lanes a particle: three warps a sub-partition (18,240 particles on 152 SMs).
+// There both forms are FP64 bound at about the same time (endpoints,
+// 200x200x20 cells, 329 steps the longest: 4864 particles 550 us against 880,
+// 9728: 629 / 947, 19456: 1020 / 979, 38912: 2317 / 1050).
+constexpr int AXES_WARPS = 12;
 
 // one axis of a cell's record
 struct AxisRec {
@@ -1239,7 +1239,10 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s)
 cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_total <= 0) return cudaSuccess;
-    const bool few = b.n_total <= AXES_MAX;
+    int sms = 0;
+    const cudaError_t err = sm_count(&sms);
+    if (err != cudaSuccess) return err;
+    const bool few = few_particles(b.n_total, AXES_WARPS, sms);
     if (b.n_reqs == 1) {
         const F64Engine<true> e{f, b};
         return few ? launch_axes(e, modes, s) : launch_tracking(e, modes, schedule, block, s);

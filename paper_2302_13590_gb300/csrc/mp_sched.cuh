@@ -327,6 +327,9 @@ __device__ __forceinline__ bool path_start(const E& e, const S& s)
 
 constexpr int AXES_PARTICLES = 10;   // of a warp whose particles have three lanes each (lanes 30 and 31 none)
 
+// n particles, three lanes each, fill at most `warps` warps on each of the SMs
+inline bool few_particles(long long n, int warps, int sms) { return n <= (long long)warps * sms * AXES_PARTICLES; }
+
 template <class E, bool TS, bool PL>
 __global__ void __launch_bounds__(256, E::min_blocks(false, TS, PL)) k_track_static(E e)
 {
@@ -438,6 +441,14 @@ __global__ void __launch_bounds__(256, E::min_blocks(true, TS, PL)) k_track_dyna
     window_end(e);
 }
 
+// the multiprocessors of the current device
+inline cudaError_t sm_count(int* sms)
+{
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 // One variant of the tracking kernel: opt in to more than 48 KB of dynamic
 // shared memory when the queues need it, size a persistent grid by occupancy.
 // (the queues of a block follow one another in dynamic shared memory: each
@@ -455,9 +466,8 @@ cudaError_t launch_variant(E e, int schedule, int block, size_t smem, cudaStream
     }
     long long grid = (e.b.n_total + block - 1) / block;
     if (schedule != MP_SCHED_STATIC) {
-        int dev = 0, sms = 0, per_sm = 0;
-        if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
-        if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
+        int sms = 0, per_sm = 0;
+        if ((err = sm_count(&sms)) != cudaSuccess) return err;
         if ((err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem)) != cudaSuccess)
             return err;
         if (per_sm < 1) per_sm = 1;
@@ -503,9 +513,8 @@ cudaError_t launch_tracking(const E& e, unsigned modes, int schedule, int block,
         // spread evenly over the SMs (60,000 particles, FP64: 12 or 16 warps an
         // SM in blocks of 128, 13 in blocks of 32: 1.69 against 1.44 ms), and
         // for rounds of any number of warps.
-        int dev = 0, sms = 0;
-        cudaError_t err = cudaGetDevice(&dev);
-        if (err == cudaSuccess) err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        int sms = 0;
+        const cudaError_t err = sm_count(&sms);
         if (err != cudaSuccess) return err;
         block = (E::EVEN_ROUNDS && schedule != MP_SCHED_STATIC) || e.b.n_total <= 512LL * sms ? 32 : 128;
     }
