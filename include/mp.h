@@ -417,8 +417,8 @@ typedef struct {
  * 64/128/256 x steps per fetch 1/4/16 for dynamic) on the first
  * min(n, sample) particles of the group (sample <= 0: all of them) with
  * options o (the group is not changed), keep the fastest in the context for (field, o->precision,
- * timeseries or not) and return it; later requests with MP_SCHED_AUTO use
- * it.  Synchronous (bounded waits).  The paper's scheduling study (Results,
+ * timeseries or not) while the field is loaded and return it; later requests
+ * with MP_SCHED_AUTO use it.  Synchronous (bounded waits).  The paper's scheduling study (Results,
  * "Thread scheduling") is this choice made by measurement.
  * Errors: as mp_track, MP_ERR_TIMEOUT. */
 /* Passage: Results, "Thread scheduling" (the schedule chosen by measurement). */

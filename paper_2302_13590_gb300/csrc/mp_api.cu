@@ -629,6 +629,9 @@ int mp_field_free(mp_field* f)
         }
         ctx->ended.clear();
         ctx->fields.erase(f);
+        // (its tuned launches go with it: a later field may get its address)
+        for (auto it = ctx->tuned.begin(); it != ctx->tuned.end();)
+            it = it->first.f == f ? ctx->tuned.erase(it) : std::next(it);
     }
     if (e == cudaSuccess && f->na_used) e = cudaStreamWaitEvent(ctx->load_st, f->na_ev, 0);
     if (e != cudaSuccess || f->foreign) {
