@@ -1764,6 +1764,17 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
     mp_track_opts oo = *o;
     oo.flags &= ~MP_TRACK_UPDATE_GROUP;
     oo.schedule = MP_SCHED_DYNAMIC;
+    // A sample of few particles runs as three lanes a particle whatever is
+    // named: there is nothing to choose, and its times say nothing about the
+    // launches that a choice would shape.
+    mp::LaunchForm form{};
+    const long long timed = sample > 0 ? std::min<long long>(sample, g->n) : g->n;
+    MP_CUDA(g->field->usg                          ? mp::form_usg(timed, &form)
+            : o->precision == MP_PREC_FP64         ? mp::form_fp64(timed, &form)
+            : o->precision == MP_PREC_MIXED        ? mp::form_mixed(timed, &form)
+                                                   : mp::form_mixed_f64t(timed, &form),
+            "mp_autotune");
+    if (form.few) cands.assign(1, {MP_SCHED_DYNAMIC, form.block, form.fetch});
     mp_tuning best{};
     best.ms = INFINITY;
     unsigned modes = 0;
@@ -1791,7 +1802,7 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
         }
     }
     best.tried = (int32_t)cands.size();
-    {
+    if (!form.few) {
         std::lock_guard<std::mutex> lk(ctx->mu);
         ctx->tuned[TuneKey{g->field, o->precision, (modes & mp::MODE_TS) ? 1 : 0}] = best;
     }

@@ -1236,6 +1236,8 @@ cudaError_t launch_spread_window(const Batch& b, cudaStream_t s)
     return cudaGetLastError();
 }
 
+cudaError_t form_fp64(long long n, LaunchForm* out) { return form_of<F64Engine<true>>(n, AXES_WARPS, out); }
+
 cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_total <= 0) return cudaSuccess;

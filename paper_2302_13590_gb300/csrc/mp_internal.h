@@ -301,6 +301,16 @@ cudaError_t launch_release_explicit(const DevField& f, const DevState& st, long 
 // ts: true if any request of the batch writes timeseries records
 cudaError_t launch_track_fp64(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
 cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s);
+// how a launch of n particles runs on the current device when nothing is named
+struct LaunchForm {
+    bool few;    // three lanes a particle, whatever schedule, block or fetch is named
+    int block;   // dynamic schedule: threads a block, steps a fetch
+    int fetch;
+};
+cudaError_t form_fp64(long long n, LaunchForm* out);
+cudaError_t form_mixed(long long n, LaunchForm* out);
+cudaError_t form_mixed_f64t(long long n, LaunchForm* out);
+cudaError_t form_usg(long long n, LaunchForm* out);
 // zero the counters of a batch's requests (n_reqs > 1)
 cudaError_t launch_zero_counters(const Batch& b, cudaStream_t s);
 // copy the first request's launch window into the other requests of a batch

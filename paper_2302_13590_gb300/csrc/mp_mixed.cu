@@ -12,6 +12,8 @@ namespace mp {
 // wait for one FP64 unit).
 constexpr int MIXED_AXES_WARPS = 20;
 
+cudaError_t form_mixed(long long n, LaunchForm* out) { return form_of<MixEngine<false, true>>(n, MIXED_AXES_WARPS, out); }
+
 cudaError_t launch_track_mixed(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_total <= 0) return cudaSuccess;

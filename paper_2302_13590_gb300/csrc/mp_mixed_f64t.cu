@@ -6,6 +6,8 @@
 
 namespace mp {
 
+cudaError_t form_mixed_f64t(long long n, LaunchForm* out) { return form_of<MixEngine<true, true>>(n, 0, out); }
+
 cudaError_t launch_track_mixed_f64t(const DevField& f, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_reqs == 1)

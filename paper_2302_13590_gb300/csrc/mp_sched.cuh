@@ -21,6 +21,8 @@
 // Per-status counts and cell-step totals (the paper's `reduction` counters,
 // Fig. 2) go to shared-memory atomics and one global atomic per block.
 #pragma once
+#include <climits>
+
 
 #include <math_constants.h>
 
@@ -504,19 +506,40 @@ cudaError_t launch_variant(E e, int schedule, int block, size_t smem, cudaStream
     return cudaGetLastError();
 }
 
+// The block of a launch whose caller names none.  One warp a block while all
+// particles fit at once: the blocks then spread evenly over the SMs (60,000
+// particles, FP64: 12 or 16 warps an SM in blocks of 128, 13 in blocks of 32:
+// 1.69 against 1.44 ms), and for rounds of any number of warps.
+template <class E>
+int default_block(long long n, int schedule, int sms)
+{
+    return (E::EVEN_ROUNDS && schedule != MP_SCHED_STATIC) || n <= 512LL * sms ? 32 : 128;
+}
+
+// How the dynamic schedule runs n particles when the caller names nothing
+// (few_warps: the engine's limit of the few-particle form, 0: it has none; that
+// form has no block or fetch to choose, so these are a larger launch's).
+template <class E>
+cudaError_t form_of(long long n, int few_warps, LaunchForm* out)
+{
+    int sms = 0;
+    const cudaError_t err = sm_count(&sms);
+    if (err != cudaSuccess) return err;
+    out->few = few_particles(n, few_warps, sms);
+    out->block = default_block<E>(out->few ? LLONG_MAX : n, MP_SCHED_DYNAMIC, sms);
+    out->fetch = E::FETCH;
+    return cudaSuccess;
+}
+
 template <class E>
 cudaError_t launch_tracking(const E& e, unsigned modes, int schedule, int block, cudaStream_t st)
 {
     if (e.b.n_total <= 0) return cudaSuccess;
     if (block <= 0) {
-        // One warp a block while all particles fit at once: the blocks then
-        // spread evenly over the SMs (60,000 particles, FP64: 12 or 16 warps an
-        // SM in blocks of 128, 13 in blocks of 32: 1.69 against 1.44 ms), and
-        // for rounds of any number of warps.
         int sms = 0;
         const cudaError_t err = sm_count(&sms);
         if (err != cudaSuccess) return err;
-        block = (E::EVEN_ROUNDS && schedule != MP_SCHED_STATIC) || e.b.n_total <= 512LL * sms ? 32 : 128;
+        block = default_block<E>(e.b.n_total, schedule, sms);
     }
     if (block > 256) block = 256;
     block = (block + 31) / 32 * 32;

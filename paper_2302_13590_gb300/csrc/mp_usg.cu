@@ -623,6 +623,8 @@ struct UsgEngine {
     }
 };
 
+cudaError_t form_usg(long long n, LaunchForm* out) { return form_of<UsgEngine<true>>(n, 0, out); }
+
 cudaError_t launch_track_usg(const DevUsg& u, const Batch& b, unsigned modes, int schedule, int block, cudaStream_t s)
 {
     if (b.n_reqs == 1) return launch_tracking(UsgEngine<true>{u, b}, modes, schedule, block, s);

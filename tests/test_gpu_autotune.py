@@ -1,5 +1,6 @@
-"""What mp_autotune and mp_set_tuning keep: nothing beyond the field that it
-belongs to."""
+"""What mp_autotune keeps: nothing from a sample that every candidate tracks
+with the same few-particle kernel, and nothing beyond the field it was measured
+on."""
 import numpy as np
 import pytest
 
@@ -27,6 +28,23 @@ def _ms(ctx, gh, precision, schedule, reps=1):
         out.append(r.stats()["kernel_ms"])
         r.free()
     return float(np.median(out))
+
+
+@pytest.mark.parametrize("precision,few", [(mp.PREC_FP64, 18240), (mp.PREC_MIXED, 30400)])
+@pytest.mark.parametrize("sample", [False, True])
+def test_few_particles_store_nothing(ctx, precision, few, sample):
+    w = I.workload("cfg1")
+    fh = ctx.field(w.field)
+    n = few if not sample else 40000
+    gh = ctx.release_box(fh, n, w.release.lo, w.release.hi, 5)
+    many = ctx.release_box(fh, 40000, w.release.lo, w.release.hi, 6)
+    mp.mp_set_tuning(ctx.h, fh, precision, False, SLOW)
+    assert _ms(ctx, many, precision, mp.SCHED_AUTO) > 20.0
+    t = mp.mp_autotune(ctx.h, gh, mp.make_opts(precision=precision), sample=1000 if sample else 0)
+    assert t["tried"] == 1 and t["ms"] > 0.0 and 32 <= t["block"] <= 256
+    assert _ms(ctx, many, precision, mp.SCHED_AUTO) > 20.0
+    mp.mp_set_tuning(ctx.h, fh, precision, False, t)      # the result is one that can be installed
+    assert _ms(ctx, many, precision, mp.SCHED_AUTO) < 20.0
 
 
 def test_tuning_goes_with_its_field(ctx):
