@@ -417,12 +417,15 @@ typedef struct {
     float ms;                 /* best time of the timed sample */
 } mp_tuning;
 
-/* Time candidate launch configurations (static and dynamic schedule x block
- * 64/128/256 x steps per fetch 1/4/16 for dynamic) on the first
+/* Time candidate launch configurations (what MP_SCHED_AUTO launches without a
+ * tuning; static and dynamic schedule x block 64/128/256 x steps per fetch
+ * 1/4/16 for dynamic) on the first
  * min(n, sample) particles of the group (sample <= 0: all of them) with
  * options o (the group is not changed), keep the fastest in the context for (field, o->precision,
  * timeseries or not) while the field is loaded and return it; later requests
- * with MP_SCHED_AUTO use it.  A sample small enough for three lanes a particle
+ * with MP_SCHED_AUTO use it.  When no candidate gains 0.5 % over the launch
+ * without a tuning, that one stays, chosen by size as before, and its shape at
+ * this size is returned.  A sample small enough for three lanes a particle
  * (see MP_SCHED_STATIC) leaves nothing to choose: one launch is timed, nothing
  * is kept, and the shape that a larger launch takes by itself is returned.
  * Synchronous (bounded waits).  The paper's scheduling study (Results,

@@ -1757,7 +1757,7 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
     MP_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     struct Cand { int sched, block, spf; };
-    std::vector<Cand> cands;
+    std::vector<Cand> cands{{MP_SCHED_DYNAMIC, 0, 0}};   // first what is launched without a tuning
     for (int b : {64, 128, 256}) cands.push_back({MP_SCHED_STATIC, b, 0});
     for (int b : {64, 128, 256})
         for (int spf : {1, 4, 16}) cands.push_back({MP_SCHED_DYNAMIC, b, spf});
@@ -1774,7 +1774,7 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
             : o->precision == MP_PREC_MIXED        ? mp::form_mixed(timed, &form)
                                                    : mp::form_mixed_f64t(timed, &form),
             "mp_autotune");
-    if (form.few) cands.assign(1, {MP_SCHED_DYNAMIC, form.block, form.fetch});
+    if (form.few) cands.resize(1);
     mp_tuning best{};
     best.ms = INFINITY;
     unsigned modes = 0;
@@ -1794,7 +1794,8 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
         if (r->seq) end_request(r);
         else drop_request(r);
         if (rc != MP_OK) return rc;
-        if (ci > 0 && ms < best.ms) {
+        // (another launch has to gain more than large ones differ by from run to run)
+        if (ci > 0 && ms < best.ms * (best.block == 0 ? 0.995f : 1.0f)) {
             best.ms = ms;
             best.schedule = c.sched;
             best.block = c.block;
@@ -1803,8 +1804,14 @@ int mp_autotune(mp_ctx* ctx, mp_group* g, const mp_track_opts* o, int64_t sample
     }
     best.tried = (int32_t)cands.size();
     if (!form.few) {
+        const TuneKey key{g->field, o->precision, (modes & mp::MODE_TS) ? 1 : 0};
         std::lock_guard<std::mutex> lk(ctx->mu);
-        ctx->tuned[TuneKey{g->field, o->precision, (modes & mp::MODE_TS) ? 1 : 0}] = best;
+        if (best.block == 0) ctx->tuned.erase(key);   // (the launch chosen by size is the best)
+        else ctx->tuned[key] = best;
+    }
+    if (best.block == 0) {
+        best.block = form.block;
+        best.steps_per_fetch = form.fetch;
     }
     *out = best;
     return MP_OK;

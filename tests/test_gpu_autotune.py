@@ -1,6 +1,6 @@
 """What mp_autotune keeps: nothing from a sample that every candidate tracks
-with the same few-particle kernel, and nothing beyond the field it was measured
-on."""
+with the same few-particle kernel, never a launch slower than the one chosen
+without it, and nothing beyond the field it was measured on."""
 import numpy as np
 import pytest
 
@@ -45,6 +45,20 @@ def test_few_particles_store_nothing(ctx, precision, few, sample):
     assert _ms(ctx, many, precision, mp.SCHED_AUTO) > 20.0
     mp.mp_set_tuning(ctx.h, fh, precision, False, t)      # the result is one that can be installed
     assert _ms(ctx, many, precision, mp.SCHED_AUTO) < 20.0
+
+
+@pytest.mark.parametrize("precision", [mp.PREC_FP64, mp.PREC_MIXED])
+def test_tuned_is_not_slower_than_untuned(ctx, precision):
+    f = I.random_box_field(20, 100, 100, seed=5, lnk_var=1.0, n_wells=4)
+    fh = ctx.field(f)
+    cells, frac = I.explicit_particles(f, 60000, seed=3, cols=(1, 5))
+    gh = ctx.release_explicit(fh, cells, frac)
+    untuned = _ms(ctx, gh, precision, mp.SCHED_DYNAMIC, 9)
+    t = mp.mp_autotune(ctx.h, gh, mp.make_opts(precision=precision))
+    assert t["tried"] == 13
+    tuned = _ms(ctx, gh, precision, mp.SCHED_AUTO, 9)
+    # (medians of nine launches lie within 1 % of each other)
+    assert tuned <= 1.02 * untuned, (tuned, untuned, t)
 
 
 def test_tuning_goes_with_its_field(ctx):
