@@ -564,8 +564,8 @@ int mp_track_launches(const mp_track_opts* o, int32_t* launches);
  * else chunks of about 128 K particles, at most 16 of them).  Chunk c's
  * copy-in, release and tracking run in order on the second of two internal
  * streams when c is odd, the first otherwise, and its copy-out on a third:
- * every chunk is launched before the first result is read, and the result
- * copies of one chunk overlap the tracking of the next.  MP_SCHED_AUTO runs the chunks
+ * three chunks are launched ahead of the one whose results are read, and the
+ * result copies of one chunk overlap the tracking of the next.  MP_SCHED_AUTO runs the chunks
  * with the static schedule (its blocks retire as their particles finish, so
  * the next chunk's blocks take their SMs).  The results are those of one
  * mp_release_group + mp_track + mp_get_endpoints / mp_get_timeseries over

@@ -1604,9 +1604,12 @@ int mp_track_host(mp_ctx* ctx, const mp_field* f, int64_t n, const int32_t* cell
     MP_CUDA(cudaSetDevice(ctx->device), "cudaSetDevice");
     // Chunks of at most 128 K particles (up to 16 of them) unless the caller
     // says; one chunk while that is as fast or faster: a second one adds its
-    // longest path, and hides a copy that is short against FP64 tracking
-    // (20,000 particles in FP64 1.5 ms as one chunk, 1.8 as two; 200,000: 5.36
-    // and 5.78; mixed precision, 200,000: 2.11 and 1.76).
+    // longest path, and hides a copy that is short against FP64 tracking.  One
+    // chunk and two, without output times and with 10, into pinned arrays: FP64
+    // 100,000 particles 2.92 / 3.24 and 3.18 / 3.75 ms, 200,000 4.84 / 5.67 and
+    // 5.59 / 6.15, 262,144 6.43 / 7.25 and 7.20 / 6.99; mixed precision 100,000
+    // 0.90 / 0.79 and 1.16 / 1.23, 131,072 0.95 / 1.01 and 1.46 / 1.27, 200,000
+    // 1.55 / 1.36 and 2.06 / 1.61.
     const long long alone = o->precision == MP_PREC_FP64 ? 262144 : 131072;
     long long nc = n_chunks > 0 ? n_chunks : n <= alone ? 1 : std::min<long long>(16, (n + 131071) / 131072);
     nc = std::min<long long>(nc, n);
@@ -1637,12 +1640,16 @@ int mp_track_host(mp_ctx* ctx, const mp_field* f, int64_t n, const int32_t* cell
         cu(cudaEventRecord(ev_start, st[0]), "mp_track_host: event") &&
         cu(cudaStreamWaitEvent(st[1], ev_start, 0), "mp_track_host: event") &&
         cu(cudaStreamWaitEvent(st[2], ev_start, 0), "mp_track_host: event");
-    // Every chunk is uploaded and launched before the first result is read: a
-    // copy to pageable host memory blocks the caller until it is done, and
-    // between two chunks' launches it would leave the GPU idle (200,000
-    // particles, 10 output times, two chunks: 6.20 -> 5.78 ms in FP64, 2.45 ->
-    // 1.76 in mixed precision).
-    for (long long c = 0; c < nc && rc == MP_OK; ++c) {
+    // A few chunks are uploaded and launched ahead of the one whose results are
+    // read.  A copy to pageable host memory blocks the caller until it is done,
+    // and between two chunks' launches it would leave the GPU idle; a launch
+    // takes the caller 0.05 ms for 125,000 particles (it looks their positions
+    // over), and all of them before the first read would leave the copies idle.
+    // 1e6 particles, 50 output times, 8 chunks, mixed precision and FP64, into
+    // pinned arrays: ahead by one 10.5 and 25.8 ms, by three 10.5 and 25.7, by
+    // all 10.9 and 25.7; into pageable ones 18.2 and 41.6, by two 12.5 and
+    // 26.9, by three 12.3 and 25.7, by all 14.3 and 28.9.
+    auto launch = [&](long long c) {
         const long long off = c * m, cnt = std::min<long long>(m, n - off);
         cudaStream_t s = st[c & 1];
         mp_release_desc rd{};
@@ -1653,17 +1660,18 @@ int mp_track_host(mp_ctx* ctx, const mp_field* f, int64_t n, const int32_t* cell
         rd.local = local + 3 * off;
         rd.t0 = t0 ? t0 + off : nullptr;
         mp_group* g = nullptr;
-        if ((rc = mp_release_group(ctx, f, &rd, s, &g)) != MP_OK) break;
+        if ((rc = mp_release_group(ctx, f, &rd, s, &g)) != MP_OK) return;
         groups.push_back(g);
         mp_req id = 0;
-        if ((rc = mp_track(ctx, g, &oc, s, &id)) != MP_OK) break;
-        ids.push_back(id);
-    }
-    for (size_t c = 0; c < ids.size() && rc == MP_OK; ++c) {
-        Request* r = find_req(ctx, ids[c]);
+        if ((rc = mp_track(ctx, g, &oc, s, &id)) == MP_OK) ids.push_back(id);
+    };
+    constexpr long long AHEAD = 3;
+    for (long long c = 0; c < std::min(nc, AHEAD) && rc == MP_OK; ++c) launch(c);
+    for (long long c = 0; c < nc && rc == MP_OK; ++c) {
+        Request* r = find_req(ctx, ids[(size_t)c]);
         cudaStream_t s = st[2];
         if (!cu(cudaStreamWaitEvent(s, r->k1, 0), "mp_track_host: event")) break;
-        const size_t u = (size_t)r->n, q = c * (size_t)m;
+        const size_t u = (size_t)r->n, q = (size_t)(c * m);
         struct { void* dst; const void* src; size_t bytes; } cp[] = {
             {ep->cell ? ep->cell + q : nullptr, r->d.cell, 4 * u},
             {ep->x ? ep->x + q : nullptr, r->d.x, 8 * u},
@@ -1685,6 +1693,7 @@ int mp_track_host(mp_ctx* ctx, const mp_field* f, int64_t n, const int32_t* cell
             cu(cudaMemcpy2DAsync(ts + q, sizeof(mp_ts_record) * (size_t)n, r->d.ts, sizeof(mp_ts_record) * u,
                                  sizeof(mp_ts_record) * u, (size_t)r->n_times, cudaMemcpyDeviceToHost, s),
                "mp_track_host: timeseries copy");
+        if (rc == MP_OK && c + AHEAD < nc) launch(c + AHEAD);
     }
     // wait (bounded) for the last copy; after an error, for what was started
     if (rc == MP_OK && cu(cudaEventRecord(ev_end, st[2]), "mp_track_host: event")) rc = wait_event(ev_end, -1);
