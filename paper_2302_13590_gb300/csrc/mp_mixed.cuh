@@ -45,8 +45,9 @@ template <bool F64T, bool ONE_REQ>
 struct MixEngine {
     static constexpr bool ONE = ONE_REQ;
     static constexpr bool OWN_SLOTS = true;   // records wait in the lane's own slots
-    static constexpr bool EVEN_ROUNDS = false;   // (issue bound: as many warps as fit)
-    static constexpr int FETCH = 16;          // steps per fetch
+    // (issue bound: as many warps as fit; with FP64 time the FP64 pipe binds)
+    static constexpr bool EVEN_ROUNDS = F64T;
+    static constexpr int FETCH = F64T ? 4 : 16;   // steps per fetch
     // What bounds it: issue (70 % of the slots; ALU instructions take two
     // cycles each), with 32 warps an SM hiding the rest, so four blocks of 256
     // threads at 64 registers and nothing spilled.  For that the state is kept
@@ -60,7 +61,19 @@ struct MixEngine {
     // kernel keeps 80 registers (the descriptors are read through a table):
     // three blocks; 240,000 particles of 24 requests 1.07 ms, at 64 registers
     // and four blocks 1.14.
-    static constexpr int min_blocks(bool dynamic, bool, bool pl) { return pl ? 0 : (dynamic ? (ONE ? 4 : 3) : 4); }
+    // With FP64 time (F64T) three log1p a step on the FP64 pipe bind it, as the
+    // FP64 engine is bound: an idle lane costs as much as a live one, warps
+    // beyond 16 an SM gain nothing, and registers are there.  So its persistent
+    // kernel takes two blocks, even rounds and 4 steps a fetch (1e6 particles,
+    // 50 output times 104.2 -> 101.7 ms with the constants above against these,
+    // endpoints 99.3 -> 96.1; 200,000 24.3 -> 22.2 and 22.7 -> 21.2; 100,000
+    // with pathlines and output times 13.3 -> 11.5), its static one with both
+    // three blocks (13.5 -> 13.2).
+    static constexpr int min_blocks(bool dynamic, bool ts, bool pl)
+    {
+        if (F64T && (dynamic || (ts && pl))) return dynamic ? 2 : 3;
+        return pl ? 0 : (dynamic ? (ONE ? 4 : 3) : 4);
+    }
     DevField f;
     Batch b;
 
