@@ -67,11 +67,15 @@ struct MixEngine {
     // kernel takes two blocks, even rounds and 4 steps a fetch (1e6 particles,
     // 50 output times 104.2 -> 101.7 ms with the constants above against these,
     // endpoints 99.3 -> 96.1; 200,000 24.3 -> 22.2 and 22.7 -> 21.2; 100,000
-    // with pathlines and output times 13.3 -> 11.5), its static one with both
-    // three blocks (13.5 -> 13.2).
+    // with pathlines and output times 13.3 -> 11.5).
+    // Kernels with pathlines and output times take three blocks, 80 registers:
+    // without a target the compiler spills at 64 (100,000 particles of ten
+    // requests 1.34 -> 1.15 ms, static 1.20 -> 1.11; one request 1.06 -> 1.05;
+    // with FP64 time, static, 13.5 -> 13.2).
     static constexpr int min_blocks(bool dynamic, bool ts, bool pl)
     {
-        if (F64T && (dynamic || (ts && pl))) return dynamic ? 2 : 3;
+        if (F64T && dynamic) return 2;
+        if (ts && pl) return 3;
         return pl ? 0 : (dynamic ? (ONE ? 4 : 3) : 4);
     }
     DevField f;
