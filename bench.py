@@ -588,7 +588,7 @@ def run_ours(args):
             r.free()
         mp.mp_group_free(gh)
         f64t = {"cell_steps_per_s": st["cell_steps"] / (np.mean(kms) / 1e3), "kernel_ms": float(np.mean(kms)),
-                "what": "FP64 cumulative time and FP64 log1p(z)/z near z = 0; dynamic schedule, 128 threads"}
+                "what": "FP64 cumulative time and FP64 log1p(z)/z near z = 0; dynamic schedule, block and fetch chosen at launch"}
 
     # end to end through the C ABI with host buffers (mp_track_host): pinned host release
     # arrays in, endpoint and timeseries records out, every step
@@ -632,7 +632,8 @@ def run_ours(args):
             # quarter
             for _ in range(max(args.steps, 10)):
                 # one call: chunked release + tracking on two streams, result
-                # copies of one chunk overlapping the tracking of the next
+                # copies of one chunk on a third, overlapping the tracking of
+                # the next
                 tc = time.perf_counter()
                 _, _, st = mp.mp_track_host(ctx.h, fh, cells_h, local_h, opts, n_chunks=args.e2e_chunks,
                                             out=ep_host, ts_out=ts_host)
@@ -645,7 +646,7 @@ def run_ours(args):
         e2e = {"value": e2e_vals["fp64"], "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                "mixed": e2e_vals["mixed"], "calls": max(args.steps, 10),
                "ms_per_call": {"fp64": e2e_vals["fp64_ms_per_call"], "mixed": e2e_vals["mixed_ms_per_call"]},
-               "call": "mp_track_host: pinned host arrays in and out; chunks on two streams, copies overlapped"}
+               "call": "mp_track_host: pinned host arrays in and out; chunks tracked on two streams, copied back on a third"}
 
     if rank != 0:
         ctx.close()

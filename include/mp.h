@@ -599,18 +599,18 @@ int mp_track_host(mp_ctx* ctx, const mp_field* f, int64_t n, const int32_t* cell
  * timeseries mode, the [n_times][n] record buffer (device).  times stays a
  * host array.  The call allocates nothing: no cudaMalloc, cudaFree or
  * allocating library routine.  Its only other device memory is a fixed
- * file-scope array of 8 + 13 + 2 * MP_NOALLOC_MAX_TIMES 64-bit words plus
- * the launch's request descriptor (queue head, counters, the output times in
- * FP64 and as FP32 pairs; about 66 KB) that every GPU that loads the library
- * holds until the process exits.
+ * file-scope array of 8 + 13 + 2 * MP_NOALLOC_MAX_TIMES 64-bit words (queue
+ * head, counters, the output times in FP64 and as FP32 pairs; about 66 KB)
+ * that every GPU that loads the library holds until the process exits.
  *   - The call runs on the device of f's context and restores the caller's
  *     current device before it returns.
  *   - The first call on each device takes the array's device address
  *     (cudaGetSymbolAddress) and keeps it.
- *   - The output times and the request descriptor reach the device through
- *     cudaMemcpyAsync from pageable host memory, which may block the calling
- *     thread until `stream` reaches the copy.  A stream that is capturing is
- *     refused (MP_ERR_INVALID_ARG).
+ *   - The output times reach the device through cudaMemcpyAsync from pageable
+ *     host memory, which may block the calling thread until `stream` reaches
+ *     the copy.  A stream that is capturing is refused (MP_ERR_INVALID_ARG).
+ *   - The offsets are taken as they are: one outside its cell (rounded, say)
+ *     makes the exit time to the face behind it negative.
  *   - Every call shares the array, which keeps the last call's contents; the
  *     call clears the queue head and counters itself.  Calls that overlap on
  *     the GPU (different streams, or a second call before the first has run)

@@ -907,12 +907,16 @@ struct F64Engine {
 // smallest FP32 estimate (so that a lane that cannot win never sends the warp
 // into log1p's general form), then on the smallest exact time, by shuffles;
 // the next cell's record is read while the axes move; and everything but
-// crossing into the next cell is one rare branch, run on the group's first
-// lane with the axes gathered through the one-lane engine's own functions.
-// Every particle has its lanes from the start, so the schedules would give
-// the same.  One step of 4864 particles 2.7 -> 1.7 us; 1000 particles, 50x50
-// cells 135 -> 93 us; 5003 pathlines, 7x61x83 cells 449 -> 277 us; 10,000
-// particles to a stop time, 200x200x20 cells 772 -> 491 us.
+// crossing into the next cell is one rare branch of the warp, in which the
+// group's lanes each end or move their axis and its first lane writes records,
+// points and ends, with the axes gathered, through the one-lane engine's own
+// functions.  Every particle has its lanes from the start, so the schedules
+// would give the same.  One step of 4864 particles 2.7 -> 1.7 us; 1000
+// particles, 50x50 cells 135 -> 93 us; 5003 pathlines, 7x61x83 cells 449 ->
+// 277 us; 10,000 particles to a stop time, 200x200x20 cells 772 -> 491 us.
+// (The range check of the next cell and the signed choice of the axis came
+// later: 4000 particles, endpoints 553 us before both, 545 with the choice in
+// a step of its own, 549 with the check.)
 // Launches of up to this many warps of ten particles on each SM take three
 // lanes a particle: three warps a sub-partition (18,240 particles on 152 SMs).
 // There both forms are FP64 bound at about the same time (endpoints,

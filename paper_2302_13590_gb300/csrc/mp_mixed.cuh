@@ -574,9 +574,10 @@ struct MixEngine {
 // 3 g + a of a warp holds axis a of its particle g: one exit time and one
 // motion a lane, the smallest time agreed by shuffles, the next cell's record
 // read while the axes move, and everything but crossing into the next cell in
-// one branch, on the group's first lane with the axes gathered.  One step of
-// 4864 particles 0.83 -> 0.42 us; 4000 particles with 20 output times,
-// 200x200x20 cells 391 -> 198 us.
+// one branch of the warp, in which the group's first lane writes records,
+// points and ends with the axes gathered.  One step of 4864 particles 0.83 ->
+// 0.42 us; 4000 particles with 20 output times, 200x200x20 cells 391 -> 195
+// us (198 with the range check of the next cell).
 template <bool ONE, bool TS, bool PL>
 __global__ void __launch_bounds__(32) k_track_axes_mixed(MixEngine<false, ONE> e)
 {

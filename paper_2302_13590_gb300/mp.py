@@ -449,7 +449,8 @@ def mp_get_stats(ctx, req: int) -> dict:
 
 
 def mp_track_host(ctx, fh, cell, local, opts: "TrackOpts", t0=None, n_chunks: int = 0, out=None, ts_out=None):
-    """Host-to-host tracking with transfers overlapped (chunked, two streams).
+    """Host-to-host tracking with transfers overlapped (in chunks: two streams
+    that track, one that copies back).
     cell (n,), local (n, 3) host arrays; out: dict of host endpoint arrays
     (None: allocated); ts_out: [n_times, n] TS_RECORD array for timeseries
     mode (None: allocated when the mode asks for it).  Returns (endpoints,
