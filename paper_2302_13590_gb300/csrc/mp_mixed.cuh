@@ -577,7 +577,7 @@ struct MixEngine {
 // one branch of the warp, in which the group's first lane writes records,
 // points and ends with the axes gathered.  One step of 4864 particles 0.83 ->
 // 0.42 us; 4000 particles with 20 output times, 200x200x20 cells 391 -> 195
-// us (198 with the range check of the next cell).
+// us (198 with the range check of the next cell in front of its load).
 template <bool ONE, bool TS, bool PL>
 __global__ void __launch_bounds__(32) k_track_axes_mixed(MixEngine<false, ONE> e)
 {
@@ -658,12 +658,18 @@ __global__ void __launch_bounds__(32) k_track_axes_mixed(MixEngine<false, ONE> e
         const int fidx = 2 * ax + (fx > 0 ? 1 : 0);
         const int cls = ax < 0 ? (int)NB_OUTSIDE : (int)((nb >> (2 * fidx)) & 3u);
         const int c2 = s.c + fx * (ax == 0 ? 1 : (ax == 1 ? stride_y : stride_z));
-        const bool inside = (unsigned)c2 < (unsigned)f.ncell;   // (false across an outer face; else an error)
+        // (its record is read whether it is entered or not, at an index held
+        // inside the grid, so that the load waits neither for the neighbour's
+        // class nor for the range check: a request of 4000 particles with 20
+        // output times 242 us without the check, 245 to 249 with the load
+        // behind it, 233 so)
+        const int at = (int)min((unsigned)c2, (unsigned)f.ncell - 1u);
+        float n1, n2;
+        unsigned nnb;
+        read(at, n1, n2, nnb);
+        const bool inside = at == c2;   // (false across an outer face; else an error)
         const bool enter =
             go && ax >= 0 && inside && (cls == NB_ACTIVE || (cls == NB_SINK && !sink_stops(p, f.sinkfrac, c2)));
-        float n1 = 0.0f, n2 = 0.0f;
-        unsigned nnb = 0;
-        if (enter) read(c2, n1, n2, nnb);
         float nh, nl;
         E::ff_add(s.th, s.tl, tmin, nh, nl);
         const float xn = E::move(A, up, x, tmin);
