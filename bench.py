@@ -64,26 +64,26 @@ BYTES_PER_STEP = {"fp64": 57.0, "mixed": 29.0}
 # the output records, both in proportion to the particle count.  Each figure
 # holds only for the kernel sources it was taken from (the hash beside it,
 # kernel_src_hash); otherwise the bench reports it as null.
-MIXED_SRC = "9ad6f4475c3fe2a1"   # mixed kernel at the capture (comments apart)
-FP64_SRC = "514402b85b379669"    # FP64 kernel at its capture (comments apart)
-TRAFFIC = {"fp64": {"src": FP64_SRC, "value": 5 * (369.524480e6 + 300.766464e6)},
-           "mixed": {"src": MIXED_SRC, "value": 5 * (37.743872e6 + 281.658624e6)}}
+MIXED_SRC = "801bede7b06dcba4"   # mixed kernel at the capture
+FP64_SRC = "753a0ea3a1da8438"    # FP64 kernel at its capture
+TRAFFIC = {"fp64": {"src": FP64_SRC, "value": 5 * (368.098560e6 + 300.675328e6)},
+           "mixed": {"src": MIXED_SRC, "value": 5 * (37.885696e6 + 281.416448e6)}}
 # From the same capture: the FP64 pipe's busy fraction in the FP64 kernel
 # (sm__pipe_fp64_cycles_active, % of peak sustained active), the executed
 # counterpart of the algorithmic fraction (which charges every axis's exit
 # time while the kernel evaluates the exact one of about 1.1 axes a step).
-FP64_PIPE_ACTIVE = {"src": FP64_SRC, "value": 0.8343}
+FP64_PIPE_ACTIVE = {"src": FP64_SRC, "value": 0.8339}
 # Warp-instructions per cell-step of the mixed kernel in the same capture
 # (smsp__inst_executed.sum / cell-steps on 2e5 particles, static schedule,
 # 128 threads): the mixed kernel is issue-bound, and its
 # issue view compares the implied issue rate with one warp-instruction per
 # clock per SM sub-partition (152 SMs x 4 x 2.07 GHz).
-MIXED_INST_PER_STEP = {"src": MIXED_SRC, "value": 1047769077.0 / 54832447.0}
+MIXED_INST_PER_STEP = {"src": MIXED_SRC, "value": 1047770672.0 / 54832447.0}
 ISSUE_PEAK_TINST = 152 * 4 * 2.07e9 / 1e12
 # L2 read bytes per cell-step in the same capture (lts__t_sectors_srcunit_tex_op_read
 # x 32 B / cell-steps): the record gather, cell sizes, output times.
-L2_READ_PER_STEP = {"fp64": {"src": FP64_SRC, "value": 269264168.0 * 32 / 54832426.0},
-                    "mixed": {"src": MIXED_SRC, "value": 62323465.0 * 32 / 54832447.0}}
+L2_READ_PER_STEP = {"fp64": {"src": FP64_SRC, "value": 269252290.0 * 32 / 54832426.0},
+                    "mixed": {"src": MIXED_SRC, "value": 62335077.0 * 32 / 54832447.0}}
 
 
 # Sources of each tracking kernel's device code: its unit and every header
